@@ -195,7 +195,7 @@ rsol_status rsol_batch_init(const rsol_params *p, const rsol_batch_desc *desc, r
             rsol::count_scratch_carve(b->count_mem, b->total_packets, nkeys, &b->count);
     }
     if (e == cudaSuccess)
-        e = cudaMalloc(&b->d_work, rsol::batch_work_words(b->total_bins) * sizeof(uint32_t));
+        e = cudaMalloc(&b->d_work, rsol::batch_work_words(b->total_bins, b->total_packets) * sizeof(uint32_t));
     if (e == cudaSuccess && p->deterministic) {
         e = cudaMalloc(&b->fx, size_t(b->total_nodes) * 8 * sizeof(long long));
         if (e == cudaSuccess)
@@ -287,7 +287,6 @@ rsol_status rsol_batch_push_gather(rsol_batch_ctx *b, const rsol_particles *P, c
     d.sm_count = b->sm_count;
     d.bin_start = b->sort.bin_start;
     d.bin = b->bin;
-    d.perm = b->sort.keys[0];  // the sort's key buffer is free until the next sort
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e = b->p.precision == 32
                         ? rsol::push_batch_f32(d, b->d_boxes, b->n_boxes, b->total_bins, b->warps, b->d_work, s)

@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(NW * 32) moments_binned_kernel(MomArgs<T> a, B
             }
     };
 
-    if (hi - lo <= sparse_bin_limit<B>()) {  // few packets: the tile would cost more than their atomics
+    if (hi - lo <= sparse_sum_limit<B>()) {  // few packets: the tile would cost more than their atomics
         for (uint32_t j = lo + threadIdx.x; j < hi; j += blockDim.x) {
             const uint32_t c = a.cell[j];
             const int ix = cell_x(c), iy = cell_y(c), iz = cell_z(c);
@@ -173,7 +173,8 @@ __global__ void __launch_bounds__(NW * 32) moments_binned_kernel(MomArgs<T> a, B
             // x (bound on one packet's moment) below 2^30; bounds per packet:
             // n: w/dx^3;  momentum: n m c |u|_max;  energy: n m c^2 gamma_max;
             // current: n |q| c
-            float gmax = tile_weight_bound<SHAPE, TE, RS, PS, NW>(hist, reinterpret_cast<float *>(stage));
+            float gmax = tile_weight_bound<SHAPE, TE, RS, PS>(
+                [&](int t) { return hist[t]; }, reinterpret_cast<float *>(stage));
             __shared__ float s_red[3][NW];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {

@@ -4,7 +4,9 @@
 // node of their stencil: the cell for CIC, the nearest node for TSC), so the
 // CTA stages the E, B tile of its bin plus a two-node halo in shared memory,
 // and deposits into a shared-memory tile that is added to the global grid
-// once at the end.  Per warp and batch of 32 packets:
+// once at the end.  FP32 (octet_cta): packets are pushed in memory order, their
+// densities staged and deposited by stencil origin.  FP64 (binned_cta), per warp
+// and batch of 32 packets:
 //   phase 1, one packet per lane: weights, gather from the tile, Boris,
 //            feedback densities, drift; the packet's stencil weights and its
 //            eight densities are staged per warp.
@@ -13,9 +15,6 @@
 //            stencil origin along the lanes (equal anchors are adjacent after
 //            the sort), accumulate W * Q in registers and add the run's sum
 //            to the tile once per run.
-// Before the batches, a histogram pass over the bin's packets sets the tile's
-// fixed-point scale and, once drift since the sort has broken the origin order,
-// a counting sort local to the CTA gives the order the batches visit.
 // Packets whose stencil leaves the tile (they drifted more than a node since
 // the sort) take the order-free path: gather from global memory and deposit
 // with global atomics.  Results equal the order-free kernel's up to the order
@@ -24,6 +23,7 @@
 
 #include <type_traits>
 
+#include "octets.cuh"
 #include "push.cuh"
 #include "tma.cuh"
 
@@ -31,12 +31,33 @@ namespace rsol {
 
 // Bins with at most this many packets skip the shared-memory tiles: staging
 // and flushing a (B + 4)^3 tile then costs more than the packets' own global
-// gathers and atomics (measured on the batch of 512 boxes, sparse bins one
-// warp each: the crossover lies near 0.45 packets per tile node).
-template <int B>
+// gathers and atomics.  Measured with 8^3 bins (sort and four steps): the batch of 512
+// boxes 24.3 ms at 768, 23.6 at 512, 23.8 at 384, 24.9 at 256; a 61 x 45 x 97 grid
+// with 1 M packets, CIC, 0.478 ms at 768 and 0.451 at 512, 384 and 256.
+// Deterministic FP32: 64-bit global atomics cost more, the crossover lies lower.
+template <typename T, int B, bool DET>
 __host__ __device__ constexpr uint32_t sparse_bin_limit()
 {
+    return sizeof(T) == 4 && DET ? 160u : B == 8 ? 512u : 256u;
+}
+
+// The same for the state moments and the adjoint step.
+template <int B>
+__host__ __device__ constexpr uint32_t sparse_sum_limit()
+{
     return B == 8 ? 768u : 256u;
+}
+
+// The same for one box's CTAs (octet_cta), where a sparse bin holds a whole CTA
+// through its packets' global atomics: 512 TSC packets of an 8^3 bin take 37 us
+// that way and 16 us through the tiles (CIC 13 and 12).  A batch's sparse bins share
+// SMs, one warp each, so its limit lies higher.  Deterministic sums round per
+// packet in one path and per run in the other: one limit, so that a batch equals
+// its boxes bit for bit.
+template <int SHAPE, int B, bool DET>
+__host__ __device__ constexpr uint32_t sparse_cta_limit()
+{
+    return DET ? sparse_bin_limit<float, B, DET>() : B == 8 ? (SHAPE == 1 ? 384u : 160u) : 128u;
 }
 
 struct BinGeom {
@@ -49,38 +70,19 @@ struct BinnedCfg {
     static constexpr int NP = SHAPE == 1 ? 2 : 3;   // stencil nodes per axis
     static constexpr int NS = NP * NP * NP;         // stencil nodes
     static constexpr int TE = B + 4;                // tile edge in nodes, origin at bin origin - 2
-    static constexpr int RS = TE;                   // row stride (dense: one bulk tensor copy)
+    static constexpr int RS = TE;                   // row stride
     static constexpr int PS = TE * RS;              // plane stride
     static constexpr int TN = TE * PS;              // tile slots
-    // deposit-tile element: 64-bit fixed point (deterministic mode), 32-bit
-    // fixed point with a per-CTA scale (FP32: native integer shared atomics are
-    // ~3.5x faster than emulated float ones), or double (FP64)
-    static constexpr bool I32 = !DET && sizeof(T) == 4;
-    using Acc = typename std::conditional<DET, long long,
-                                          typename std::conditional<I32, int, T>::type>::type;
-    // the deposit tile, and everything keyed by a packet's stencil origin (the
-    // origin histogram, the kept keys, the local sort, the run walk), has its own
-    // strides: padded so that the 27 stencil lanes of a TSC flush hit 27
-    // distinct banks with 4-byte elements (the dense field-tile strides put the
-    // z = 0 and z = 2 planes on the same banks)
-    static constexpr int DRS = sizeof(Acc) == 4 ? (TE == 12 ? 14 : (TE == 8 ? 11 : RS)) : RS;
-    static constexpr int DPS = sizeof(Acc) == 4 ? (TE == 12 ? 171 : (TE == 8 ? 89 : PS)) : PS;
-    static constexpr int DTN = TE * DPS;
-    static constexpr size_t fields_bytes = size_t(TN) * 8 * sizeof(T);   // [slot][8]: E, B, 2 unused
-    static constexpr size_t dep_bytes = size_t(DTN) * 8 * sizeof(Acc);   // [q][slot]
-    // per warp: stencil weights W[32][WS] and densities + origin QO[32][12]
+    // deposit-tile element: 64-bit fixed point (deterministic mode), or T
+    using Acc = typename std::conditional<DET, long long, T>::type;
+    static constexpr size_t fields_bytes = size_t(TN) * 8 * sizeof(T);  // [slot][8]: E, B, 2 unused
+    static constexpr size_t dep_bytes = size_t(TN) * 8 * sizeof(Acc);   // [q][slot]
+    // per warp: stencil weights W[32][WS] and densities QO[32][12]
     static constexpr int WS = NS == 27 ? 28 : NS;   // weight rows padded to 16-byte stores
-    static constexpr int QO = 12;                   // 48-byte rows: conflict-free 16-byte stores
+    static constexpr int QO = 12;                   // rows apart: fewer conflicts of the 16-byte stores
     static constexpr size_t stage_words = 32 * (WS + QO);
     static constexpr size_t stage_bytes = size_t(NW) * stage_words * sizeof(T);
-    // 32-bit fixed point: the stencil-origin key of each of the bin's first KEYCAP
-    // packets, kept from the histogram pass for the local sort
-    static constexpr int KEYCAP = I32 ? 8192 : 0;
-    static constexpr size_t key_bytes = size_t(KEYCAP) * sizeof(uint16_t);
-    // the field tile is the destination of a bulk tensor copy: 128-byte
-    // aligned, so the dynamic allocation carries up to 128 bytes of padding
-    static constexpr size_t align_pad = 128;
-    static constexpr size_t smem_bytes = align_pad + fields_bytes + dep_bytes + stage_bytes + key_bytes;
+    static constexpr size_t smem_bytes = fields_bytes + dep_bytes + stage_bytes;
 };
 
 __device__ __forceinline__ int wrap_mod(int v, int n)
@@ -94,6 +96,13 @@ __device__ __forceinline__ int wrap_once(int v, int n)
 {
     v += v < 0 ? n : 0;
     return v - (v >= n ? n : 0);
+}
+
+// First stencil node relative to the cell (axis_weights without the weights).
+template <int SHAPE, typename T>
+__device__ __forceinline__ int first_node(T f)
+{
+    return SHAPE == 1 || f >= T(0.5) ? 0 : -1;
 }
 
 // Anchor node and stencil data of one axis: returns the anchor (periodic) and
@@ -288,7 +297,7 @@ __device__ __forceinline__ void origin_cursors(const int *hist, int *cursor, int
 }
 
 // Largest total weight any node of a tile can receive from the packets counted
-// in hist (packets per tile-local stencil origin, slot z PS + y RS + x): the
+// in hist(slot) (packets per tile-local stencil origin, slot z PS + y RS + x): the
 // sum over the stencil origins around the node of (packets at the origin) x
 // (largest axis weights for that offset: CIC 1, 1; TSC 1/2, 3/4, 1/2 per
 // axis).  The weights are per-axis products, so the sum is three 3-tap passes
@@ -296,85 +305,96 @@ __device__ __forceinline__ void origin_cursors(const int *hist, int *cursor, int
 // are small integers times products of 1/2 and 3/4).  scratch holds 2 TE^3
 // floats.  Returns this thread's largest node value (reduce over the CTA);
 // ends with scratch still in use by no thread, but without a final barrier.
-template <int SHAPE, int TE, int RS, int PS, int NW>
-__device__ __forceinline__ float tile_weight_bound(const int *hist, float *scratch)
+template <int SHAPE, int TE, int RS, int PS, typename Hist>
+__device__ __forceinline__ void weight_bound_pass(int pass, Hist hist, float *scratch, float &gmax)
 {
     constexpr int NP = SHAPE == 1 ? 2 : 3;
     constexpr int TT = TE * TE * TE;
     float *g1 = scratch, *g2 = scratch + TT;  // [z][y][x], TE each
     auto tap = [](int c) { return SHAPE == 1 ? 1.f : (c == 1 ? 0.75f : 0.5f); };
-    for (int r = threadIdx.x; r < TE * TE; r += blockDim.x) {  // along x: rows (z, y)
-        const int y = r % TE, z = r / TE;
+    // the rows go to the last threads (the first warps may have other work)
+    for (int r = int(blockDim.x) - 1 - int(threadIdx.x); r < TE * TE; r += blockDim.x) {
+        const int u = r % TE, z = r / TE;  // pass 0: row (z, y = u); 1: (z, x = u); 2: (y = z, x = u)
         float h[TE];
 #pragma unroll
-        for (int x = 0; x < TE; ++x)
-            h[x] = float(hist[z * PS + y * RS + x]);
+        for (int i = 0; i < TE; ++i)
+            h[i] = pass == 0 ? float(hist(z * PS + u * RS + i)) : pass == 1 ? g1[(z * TE + i) * TE + u]
+                                                                          : g2[(i * TE + z) * TE + u];
 #pragma unroll
-        for (int x = 0; x < TE; ++x) {
+        for (int i = 0; i < TE; ++i) {
             float v = 0.f;
 #pragma unroll
             for (int c = 0; c < NP; ++c)
-                v += x >= c ? tap(c) * h[x - c] : 0.f;
-            g1[(z * TE + y) * TE + x] = v;
+                v += i >= c ? tap(c) * h[i - c] : 0.f;
+            if (pass == 0)
+                g1[(z * TE + u) * TE + i] = v;
+            else if (pass == 1)
+                g2[(z * TE + i) * TE + u] = v;
+            else
+                gmax = fmaxf(gmax, v);
         }
     }
-    __syncthreads();
-    for (int r = threadIdx.x; r < TE * TE; r += blockDim.x) {  // along y: rows (z, x)
-        const int x = r % TE, z = r / TE;
-        float h[TE];
-#pragma unroll
-        for (int y = 0; y < TE; ++y)
-            h[y] = g1[(z * TE + y) * TE + x];
-#pragma unroll
-        for (int y = 0; y < TE; ++y) {
-            float v = 0.f;
-#pragma unroll
-            for (int c = 0; c < NP; ++c)
-                v += y >= c ? tap(c) * h[y - c] : 0.f;
-            g2[(z * TE + y) * TE + x] = v;
-        }
-    }
-    __syncthreads();
+}
+template <int SHAPE, int TE, int RS, int PS, typename Hist>
+__device__ __forceinline__ float tile_weight_bound(Hist hist, float *scratch)
+{
     float gmax = 0.f;
-    for (int r = threadIdx.x; r < TE * TE; r += blockDim.x) {  // along z: rows (y, x)
-        const int x = r % TE, y = r / TE;
-        float h[TE];
-#pragma unroll
-        for (int z = 0; z < TE; ++z)
-            h[z] = g2[(z * TE + y) * TE + x];
-#pragma unroll
-        for (int z = 0; z < TE; ++z) {
-            float v = 0.f;
-#pragma unroll
-            for (int c = 0; c < NP; ++c)
-                v += z >= c ? tap(c) * h[z - c] : 0.f;
-            gmax = fmaxf(gmax, v);
-        }
-    }
+    weight_bound_pass<SHAPE, TE, RS, PS>(0, hist, scratch, gmax);
+    __syncthreads();
+    weight_bound_pass<SHAPE, TE, RS, PS>(1, hist, scratch, gmax);
+    __syncthreads();
+    weight_bound_pass<SHAPE, TE, RS, PS>(2, hist, scratch, gmax);
     return gmax;
+}
+
+// Few packets: staging and flushing the tiles would cost more than the
+// packets' own global-memory gathers and atomics.
+template <typename T, int SHAPE, bool DET>
+__device__ __forceinline__ void sparse_cta(const PushArgs<T> &a, uint32_t lo, uint32_t hi)
+{
+    int sflag = 0;
+    auto gather_global = [&](int64_t node, T F[6]) { load_node(a.fields + node * 8, F); };
+    auto deposit_global = [&](int64_t node, T W, const T Q[8]) {
+        if constexpr (DET)
+            red_node_fixed(a.fx + node * 8, W, Q, a.fx_scale);
+        else
+            red_node(a.fb + node * 8, W, Q);
+    };
+    for (uint32_t j = lo + threadIdx.x; j < hi; j += blockDim.x)
+        push_one<T, SHAPE, true>(a, int64_t(j), gather_global, deposit_global, &sflag);
+    if (sflag)
+        atomicOr(a.status, sflag);
+}
+
+// Grid offsets of the rows along each axis (periodic) of the tile of TE^3 nodes
+// from node (ox, oy, oz): the grid node of tile point (lx, ly, lz) is
+// axis[lx] + axis[TE + ly] + axis[2 TE + lz].
+template <int TE>
+__device__ __forceinline__ void tile_axes(int *axis, int ox, int oy, int oz, int nx, int ny, int nz)
+{
+    if (threadIdx.x < 3 * TE) {
+        const int ax = threadIdx.x / TE, l = threadIdx.x % TE;
+        const int o = ax == 0 ? ox : (ax == 1 ? oy : oz);
+        const int n = ax == 0 ? nx : (ax == 1 ? ny : nz);
+        const int stride = ax == 0 ? 1 : (ax == 1 ? nx : nx * ny);
+        axis[threadIdx.x] = wrap_mod(o + l, n) * stride;
+    }
 }
 
 // The work of one CTA on one bin: packets [lo, hi) of the bin whose anchors
 // were in bin (bx, by, bz) of the box described by a at the last sort.
 template <typename T, int SHAPE, int B, int NW, bool DET>
 __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, uint32_t hi,
-                                           int bx, int by, int bz,
-                                           const CUtensorMap *tmap = nullptr)
+                                           int bx, int by, int bz)
 {
     using Cfg = BinnedCfg<T, SHAPE, B, NW, DET>;
     using Acc = typename Cfg::Acc;
-    constexpr bool F2 = std::is_same<T, float>::value;  // f32x2 gather and deposit
-    constexpr int TE = Cfg::TE, RS = Cfg::RS, PS = Cfg::PS;          // field tile
-    constexpr int DRS = Cfg::DRS, DPS = Cfg::DPS, DTN = Cfg::DTN;  // deposit tile, origin keys
+    constexpr int TE = Cfg::TE, RS = Cfg::RS, PS = Cfg::PS, TN = Cfg::TN;
     constexpr int NP = Cfg::NP, NS = Cfg::NS, WS = Cfg::WS, QO = Cfg::QO;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned char *smem = smem_raw + ((Cfg::align_pad - (smem_addr(smem_raw) & (Cfg::align_pad - 1))) &
-                                      (Cfg::align_pad - 1));
+    extern __shared__ __align__(16) unsigned char smem[];
     T *sf = reinterpret_cast<T *>(smem);
     Acc *sd = reinterpret_cast<Acc *>(smem + Cfg::fields_bytes);
     T *stage = reinterpret_cast<T *>(smem + Cfg::fields_bytes + Cfg::dep_bytes);
-    uint16_t *s_key = reinterpret_cast<uint16_t *>(smem + Cfg::fields_bytes + Cfg::dep_bytes +
-                                                   Cfg::stage_bytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     T *sW = stage + warp * Cfg::stage_words;  // [32][WS]
@@ -382,63 +402,21 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
 
     if (lo >= hi)
         return;
-    if (hi - lo <= sparse_bin_limit<B>()) {
-        // few packets: staging and flushing the tiles would cost more than the
-        // packets' own global-memory gathers and atomics
-        int sflag = 0;
-        auto gather_global = [&](int64_t node, T F[6]) { load_node(a.fields + node * 8, F); };
-        auto deposit_global = [&](int64_t node, T W, const T Q[8]) {
-            if (DET)
-                red_node_fixed(a.fx + node * 8, W, Q, a.fx_scale);
-            else
-                red_node(a.fb + node * 8, W, Q);
-        };
-        for (uint32_t j = lo + threadIdx.x; j < hi; j += blockDim.x)
-            push_one<T, SHAPE, true>(a, int64_t(j), gather_global, deposit_global, &sflag);
-        if (sflag)
-            atomicOr(a.status, sflag);
+    if (hi - lo <= sparse_bin_limit<T, B, DET>()) {
+        sparse_cta<T, SHAPE, DET>(a, lo, hi);
         return;
     }
     const int ox = bx * B - 2, oy = by * B - 2, oz = bz * B - 2;
-    // A tile that does not wrap around the periodic grid on any axis is one box
-    // of the field grid: one bulk tensor copy (TMA) issued by thread 0 lands it
-    // while the threads make the origin histogram below.  FP32 only, with the
-    // tensor map the host encoded for this field grid.
     constexpr int TT = TE * TE * TE;
-    const bool tma = Cfg::I32 && tmap != nullptr && ox >= 0 && oy >= 0 && oz >= 0 &&
-                     ox + TE <= a.nx && oy + TE <= a.ny && oz + TE <= a.nz;
-    __shared__ uint64_t s_tma_bar;
-    if (tma && threadIdx.x == 0)
-        mbar_init(&s_tma_bar, 1);
     // grid offsets of the tile's rows along each axis (periodic): node of tile
     // point (lx, ly, lz) = s_axis[lx] + s_axis[TE + ly] + s_axis[2 TE + lz]
     __shared__ int s_axis[3 * TE];
-    if (threadIdx.x < 3 * TE) {
-        const int ax = threadIdx.x / TE, l = threadIdx.x % TE;
-        const int o = ax == 0 ? ox : (ax == 1 ? oy : oz);
-        const int n = ax == 0 ? a.nx : (ax == 1 ? a.ny : a.nz);
-        const int stride = ax == 0 ? 1 : (ax == 1 ? a.nx : a.nx * a.ny);
-        s_axis[threadIdx.x] = wrap_mod(o + l, n) * stride;
-    }
+    tile_axes<TE>(s_axis, ox, oy, oz, a.nx, a.ny, a.nz);
     __syncthreads();
 
-    // stage the field tile (periodic) and clear the deposit tile; track the
-    // largest |E| and, per axis a, the largest |B| across a (B with its a
-    // component removed) of the tile for the fixed-point scale
-    T e2max = T(0), bp2max[3] = {T(0), T(0), T(0)};
-    auto field_bounds = [&](const T F[6]) {
-        e2max = fmax(e2max, F[0] * F[0] + F[1] * F[1] + F[2] * F[2]);
-        const T bx2 = F[3] * F[3], by2 = F[4] * F[4], bz2 = F[5] * F[5];
-        bp2max[0] = fmax(bp2max[0], by2 + bz2);
-        bp2max[1] = fmax(bp2max[1], bx2 + bz2);
-        bp2max[2] = fmax(bp2max[2], bx2 + by2);
-    };
-    if (tma && threadIdx.x == 0) {
-        mbar_arrive_expect_tx(&s_tma_bar, uint32_t(TT * 8 * sizeof(T)));
-        tma_load_4d(sf, tmap, 0, ox, oy, oz, &s_tma_bar);
-    }
+    // stage the field tile (periodic) and clear the deposit tile
     constexpr int UF = 4;  // nodes per thread per pass: all loads issued first
-    for (int t0 = threadIdx.x; !tma && t0 < TT; t0 += UF * blockDim.x) {
+    for (int t0 = threadIdx.x; t0 < TT; t0 += UF * blockDim.x) {
         T F[UF][6];
 #pragma unroll
         for (int u = 0; u < UF; ++u) {
@@ -456,189 +434,11 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
                 const int lx = t % TE, ly = (t / TE) % TE, lz = t / (TE * TE);
                 const int slot = lz * PS + ly * RS + lx;
                 sts_node(sf + slot * 8, F[u]);
-                field_bounds(F[u]);
             }
         }
     }
-    // clear the whole deposit tile, padding slots included (the origin histogram
-    // below reads every slot)
-    for (int t = threadIdx.x; t < 8 * DTN; t += blockDim.x)
+    for (int t = threadIdx.x; t < 8 * TN; t += blockDim.x)
         sd[t] = Acc(0);
-    // 32-bit fixed point: scale_q = 2^e with (packets in bin) * Wmax * bound_q
-    // below 2^30, bound_q a bound on one packet's |Q_q| (|beta_bar| < 1):
-    //   rho: w q / dx^3;  J: rho c;  S_a: rho (|E| + |B across a|), since
-    //   |(beta_bar x B)_a| <= |beta_bar| |B with its a component removed|;
-    //   H: rho c |E| (1 + h |E|)
-    __shared__ float s_scale[8], s_iscale[8];  // 32-bit fixed point: 2^e and 2^-e per density
-    __shared__ int s_local_sorted;  // 1: phase 1 visits the packets in a.perm order
-    if (threadIdx.x == 0)
-        s_local_sorted = 0;
-    if (Cfg::I32) {
-        // packets per stencil origin (histogram in the zeroed deposit tile): a node
-        // receives from at most NS origins, so NS * (largest origin count) bounds
-        // the packets that reach any one node
-        // It also counts descents of the origin along the packet order (lanes
-        // against their left neighbour): a bin still in the order of the last
-        // global sort needs no local sort below.
-        __shared__ int s_desc;
-        if (threadIdx.x == 0)
-            s_desc = 0;
-        __syncthreads();
-        int *hist = reinterpret_cast<int *>(sd);
-        T wmax = T(0);
-        int desc = 0;
-        constexpr int U = 4;  // packets per thread per pass: all loads issued first
-        for (uint32_t jb = lo; jb < hi; jb += U * blockDim.x) {  // warp-uniform trip count
-            const uint32_t j0 = jb + threadIdx.x;
-            uint32_t cc[U];
-            T f0[U], f1[U], f2[U], ww[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const uint32_t j = j0 + uint32_t(u) * blockDim.x;
-                const bool ok = j < hi;
-                cc[u] = ok ? a.cell[j] : 0xFFFFFFFFu;
-                f0[u] = ok ? a.off0[j] : T(0);
-                f1[u] = ok ? a.off1[j] : T(0);
-                f2[u] = ok ? a.off2[j] : T(0);
-                ww[u] = ok ? a.w[j] : T(0);
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                wmax = fmax(wmax, fabs(ww[u]));
-                // out of the tile or off the grid: DTN, which sorts last
-                const int key = origin_slot<SHAPE, TE, DRS, DPS, DTN>(cc[u], f0[u], f1[u], f2[u], ox,
-                                                                      oy, oz, a.nx, a.ny, a.nz);
-                if (key < DTN)
-                    atomicAdd(&hist[key], 1);
-                {
-                    const uint32_t jr = j0 + uint32_t(u) * blockDim.x - lo;  // rank in the bin
-                    if (jr < hi - lo && jr < uint32_t(Cfg::KEYCAP))
-                        s_key[jr] = uint16_t(key);
-                }
-                const int prev = __shfl_up_sync(0xffffffffu, key, 1);
-                desc += (lane > 0 && j0 + uint32_t(u) * blockDim.x < hi && key < prev) ? 1 : 0;
-            }
-        }
-        desc = __reduce_add_sync(0xffffffffu, desc);
-        if (lane == 0 && desc)
-            atomicAdd(&s_desc, desc);
-        __syncthreads();
-        // largest weight a node can receive in total (this thread's share)
-        static_assert(Cfg::stage_bytes >= 2 * size_t(TT) * sizeof(float), "stage too small");
-        float gmax = tile_weight_bound<SHAPE, TE, DRS, DPS, NW>(hist, reinterpret_cast<float *>(stage));
-        __syncthreads();
-        // sort locally once more than one packet in 32 breaks the origin order
-        if (a.perm && s_desc * 32 > int(hi - lo)) {
-            // counting sort of the bin's packets by stencil origin (local to the
-            // CTA): the histogram gives each origin's first position, and phase 1
-            // then visits the packets origin by origin, so a phase-2 run spans
-            // a whole origin however far the packets drifted since the last
-            // global sort.  Out-of-tile and off-grid packets go last.
-            int *cursor = reinterpret_cast<int *>(stage);  // free until the batches
-            if (threadIdx.x == 0)
-                s_local_sorted = 1;
-            __shared__ int s_out;
-            origin_cursors<NW, DTN>(hist, cursor, &s_out);
-            if (hi - lo <= uint32_t(Cfg::KEYCAP)) {  // keys kept from the histogram pass
-                for (uint32_t jr = threadIdx.x; jr < hi - lo; jr += blockDim.x) {
-                    const int key = s_key[jr];
-                    const int pos = key < DTN ? atomicAdd(&cursor[key], 1) : atomicAdd(&s_out, 1);
-                    a.perm[lo + uint32_t(pos)] = lo + jr;
-                }
-            } else {
-                for (uint32_t j0 = lo + threadIdx.x; j0 < hi; j0 += U * blockDim.x) {
-                    uint32_t cc[U];
-                    T f0[U], f1[U], f2[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const uint32_t j = j0 + uint32_t(u) * blockDim.x;
-                        const bool ok = j < hi;
-                        cc[u] = ok ? a.cell[j] : 0xFFFFFFFFu;
-                        f0[u] = ok ? a.off0[j] : T(0);
-                        f1[u] = ok ? a.off1[j] : T(0);
-                        f2[u] = ok ? a.off2[j] : T(0);
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const uint32_t j = j0 + uint32_t(u) * blockDim.x;
-                        if (j >= hi)
-                            continue;
-                        const int slot = origin_slot<SHAPE, TE, DRS, DPS, DTN>(
-                            cc[u], f0[u], f1[u], f2[u], ox, oy, oz, a.nx, a.ny, a.nz);
-                        const int pos = slot < DTN ? atomicAdd(&cursor[slot], 1) : atomicAdd(&s_out, 1);
-                        a.perm[lo + uint32_t(pos)] = j;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-        for (int t = threadIdx.x; t < DTN; t += blockDim.x)
-            hist[t] = 0;
-        if (tma) {
-            // the bulk copy: wait for it (bounded), then the field bounds from the tile
-            const bool arrived = mbar_wait_bounded(&s_tma_bar, 0, kTmaWaitCycles);
-            if (!__syncthreads_and(arrived)) {
-                // report it, give the copy one more bounded wait, skip the bin
-                if (threadIdx.x == 0) {
-                    atomicOr(a.status, ST_TIMEOUT);
-                    mbar_wait_bounded(&s_tma_bar, 0, kTmaWaitCycles);
-                }
-                __syncthreads();
-                return;
-            }
-            for (int t = threadIdx.x; t < TT; t += blockDim.x) {
-                T F[6];
-                lds_node(sf + t * 8, F);
-                field_bounds(F);
-            }
-        }
-        __shared__ T s_red[5][NW];
-        __shared__ float s_gmax[NW];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            e2max = fmax(e2max, __shfl_xor_sync(0xffffffffu, e2max, o));
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-                bp2max[a] = fmax(bp2max[a], __shfl_xor_sync(0xffffffffu, bp2max[a], o));
-            wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
-            gmax = fmaxf(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
-        }
-        if (lane == 0) {
-            s_red[0][warp] = e2max;
-            s_red[1][warp] = wmax;
-            s_red[2][warp] = bp2max[0];
-            s_red[3][warp] = bp2max[1];
-            s_red[4][warp] = bp2max[2];
-            s_gmax[warp] = gmax;
-        }
-        __syncthreads();
-        if (threadIdx.x < 8) {
-            const int q = threadIdx.x;
-            const int bp = q >= 4 && q < 7 ? 2 + (q - 4) : 2;  // S_q: |B| across axis q - 4
-            T em = T(0), bm = T(0), wm = T(0);
-            float gm = 0.f;
-            for (int w = 0; w < NW; ++w) {
-                em = fmax(em, s_red[0][w]);
-                wm = fmax(wm, s_red[1][w]);
-                bm = fmax(bm, s_red[bp][w]);
-                gm = fmaxf(gm, s_gmax[w]);
-            }
-            em = Math<T>::sqrt(em);
-            bm = Math<T>::sqrt(bm);
-            const T rho = wm * fabs(a.k.qv);
-            T bound = q == 0 ? rho
-                    : q < 4  ? rho * a.k.c
-                    : q < 7  ? rho * (em + bm)
-                             : rho * a.k.c * em * (T(1) + fabs(a.k.h) * em);
-            bound *= T(gm > 1.f ? gm : 1.f);
-            int e = 30;
-            if (bound > T(0) && isfinite(bound))
-                e = 30 - int(ceilf(log2f(float(bound))));
-            e = e > 60 ? 60 : (e < -60 ? -60 : e);
-            s_scale[q] = ldexpf(1.0f, e);
-            s_iscale[q] = ldexpf(1.0f, -e);
-        }
-    }
     __syncthreads();
 
     // phase-2 lane role: stencil offset and quantity range [q0, q0 + 2 or 8)
@@ -646,7 +446,7 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
     const bool p2_active = SHAPE == 1 ? true : lane < 27;
     const int pax = off_id % NP, pay = (off_id / NP) % NP, paz = off_id / (NP * NP);
     const int q0 = SHAPE == 1 ? 2 * (lane >> 3) : 0;
-    const int lane_off = paz * DPS + pay * DRS + pax;
+    const int lane_off = paz * PS + pay * RS + pax;
 
     int flag = 0;
     // each warp walks a contiguous slice of the bin, so a run of equal stencil
@@ -661,49 +461,33 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
 #pragma unroll
     for (int q = 0; q < NQ_; ++q)
         acc[q] = T(0);
-    f32x2 acc2[NQ_ / 2];  // FP32: the densities in pairs (f32x2 arithmetic)
-#pragma unroll
-    for (int q = 0; q < NQ_ / 2; ++q)
-        acc2[q] = 0;
     auto flush_acc = [&](int origin) {
         if (p2_active && origin >= 0) {
             const int t = origin + lane_off;
-            if constexpr (F2) {
-#pragma unroll
-                for (int q = 0; q < NQ_ / 2; ++q)
-                    f2_unpack(acc2[q], acc[2 * q], acc[2 * q + 1]);
-            }
 #pragma unroll
             for (int q = 0; q < NQ_; ++q) {
                 if (DET)
-                    atomicAdd(reinterpret_cast<unsigned long long *>(&sd[(q0 + q) * DTN + t]),
+                    atomicAdd(reinterpret_cast<unsigned long long *>(&sd[(q0 + q) * TN + t]),
                               static_cast<unsigned long long>(to_fixed(acc[q] * a.fx_scale)));
-                else if (Cfg::I32)
-                    atomicAdd(reinterpret_cast<int *>(&sd[(q0 + q) * DTN + t]),
-                              __float2int_rn(float(acc[q])));  // densities staged pre-scaled
                 else
-                    atomicAdd(reinterpret_cast<T *>(&sd[(q0 + q) * DTN + t]), acc[q]);
+                    atomicAdd(reinterpret_cast<T *>(&sd[(q0 + q) * TN + t]), acc[q]);
             }
         }
     };
     // software pipeline: the packet fields of batch k+1 are loaded into
     // registers while batch k is pushed and deposited
-    // (with the local sort, position jj of the bin holds packet perm[jj])
-    const bool use_perm = Cfg::I32 && s_local_sorted != 0;
-    uint32_t n_c = 0, n_j = 0;
+    uint32_t n_c = 0;
     T n_o[3] = {T(0), T(0), T(0)}, n_u[3] = {T(0), T(0), T(0)}, n_w = T(0);
     auto prefetch = [&](uint32_t jj) {
         if (jj < w_hi) {
-            const uint32_t jp = use_perm ? a.perm[jj] : jj;
-            n_j = jp;
-            n_c = a.cell[jp];
-            n_o[0] = a.off0[jp];
-            n_o[1] = a.off1[jp];
-            n_o[2] = a.off2[jp];
-            n_u[0] = a.u0[jp];
-            n_u[1] = a.u1[jp];
-            n_u[2] = a.u2[jp];
-            n_w = a.w[jp];
+            n_c = a.cell[jj];
+            n_o[0] = a.off0[jj];
+            n_o[1] = a.off1[jj];
+            n_o[2] = a.off2[jj];
+            n_u[0] = a.u0[jj];
+            n_u[1] = a.u1[jj];
+            n_u[2] = a.u2[jj];
+            n_w = a.w[jj];
         }
     };
     prefetch(w_lo + uint32_t(lane));
@@ -713,7 +497,6 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
         T fx = n_o[0], fy = n_o[1], fz = n_o[2];
         const T u0[3] = {n_u[0], n_u[1], n_u[2]};
         const T wj = n_w;
-        const uint32_t jp = n_j;  // the packet at sorted position j
         prefetch(j + 32);
         int staged = -1;
         if (j < w_hi) {
@@ -750,46 +533,22 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
                 int kx[3], ky[3], kz[3];
                 if (in_tile) {
                     const int s0 = lz * PS + ly * RS + lx;
-                    if constexpr (F2) {
-                        // pairs {Ex, Ey}, {Ez, Bx}, {By, Bz}: a node is one 16-byte
-                        // and one 8-byte load and three paired multiply-adds
-                        f32x2 g01 = 0, g23 = 0, g45 = 0;  // +0.0f in both halves
 #pragma unroll
-                        for (int cz = 0; cz < NP; ++cz)
+                    for (int cz = 0; cz < NP; ++cz)
 #pragma unroll
-                            for (int cy = 0; cy < NP; ++cy)
+                        for (int cy = 0; cy < NP; ++cy)
 #pragma unroll
-                                for (int cx = 0; cx < NP; ++cx) {
-                                    const float W = Wk[(cz * NP + cy) * NP + cx];
-                                    const f32x2 W2 = f2_pack(W, W);
-                                    const float *p = sf + (s0 + cz * PS + cy * RS + cx) * 8;
-                                    const ulonglong2 a2 = *reinterpret_cast<const ulonglong2 *>(p);
-                                    const f32x2 b2 = *reinterpret_cast<const f32x2 *>(p + 4);
-                                    g01 = f2_fma(W2, a2.x, g01);
-                                    g23 = f2_fma(W2, a2.y, g23);
-                                    g45 = f2_fma(W2, b2, g45);
+                            for (int cx = 0; cx < NP; ++cx) {
+                                const T W = Wk[(cz * NP + cy) * NP + cx];
+                                T F[6];
+                                lds_node(sf + (s0 + cz * PS + cy * RS + cx) * 8, F);
+#pragma unroll
+                                for (int q = 0; q < 3; ++q) {
+                                    E[q] += W * F[q];
+                                    Bf[q] += W * F[3 + q];
                                 }
-                        f2_unpack(g01, E[0], E[1]);
-                        f2_unpack(g23, E[2], Bf[0]);
-                        f2_unpack(g45, Bf[1], Bf[2]);
-                    } else {
-#pragma unroll
-                        for (int cz = 0; cz < NP; ++cz)
-#pragma unroll
-                            for (int cy = 0; cy < NP; ++cy)
-#pragma unroll
-                                for (int cx = 0; cx < NP; ++cx) {
-                                    const T W = Wk[(cz * NP + cy) * NP + cx];
-                                    T F[6];
-                                    lds_node(sf + (s0 + cz * PS + cy * RS + cx) * 8, F);
-#pragma unroll
-                                    for (int q = 0; q < 3; ++q) {
-                                        E[q] += W * F[q];
-                                        Bf[q] += W * F[3 + q];
-                                    }
-                                }
-                    }
-                    staged = lz * DPS + ly * DRS + lx;
+                            }
+                    staged = s0;
                 } else {
                     axis_nodes(jx, rx, a.nx, kx);
                     axis_nodes(jy, ry, a.ny, ky);
@@ -818,11 +577,6 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
                 feedback(a.k, wj, E, Bf, b, g0, Q);
                 if (in_tile) {
                     store_wrow<WS>(sW + lane * WS, Wk);
-                    if (Cfg::I32) {  // the tile's fixed-point scale (a power of two: exact)
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            Q[q] *= T(s_scale[q]);
-                    }
                     store_q8(sQ + lane * QO, Q);
                 } else {
 #pragma unroll
@@ -846,13 +600,13 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
                     const int nx_ = drift_axis(ix, fx, s * b.u1[0], a.nx, &flag);
                     const int ny_ = drift_axis(iy, fy, s * b.u1[1], a.ny, &flag);
                     const int nz_ = drift_axis(iz, fz, s * b.u1[2], a.nz, &flag);
-                    a.cell[jp] = pack_cell(nx_, ny_, nz_);
-                    a.off0[jp] = fx;
-                    a.off1[jp] = fy;
-                    a.off2[jp] = fz;
-                    a.u0[jp] = b.u1[0];
-                    a.u1[jp] = b.u1[1];
-                    a.u2[jp] = b.u1[2];
+                    a.cell[j] = pack_cell(nx_, ny_, nz_);
+                    a.off0[j] = fx;
+                    a.off1[j] = fy;
+                    a.off2[j] = fz;
+                    a.u0[j] = b.u1[0];
+                    a.u1[j] = b.u1[1];
+                    a.u2[j] = b.u1[2];
                 } else {
                     flag |= ST_NONFINITE;
                 }
@@ -882,83 +636,37 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
             const T *wrow = sW + L * WS + off_id;
             const T *qrow = sQ + L * QO + q0;
             int p = L;
-            if constexpr (F2) {
-                // densities in pairs: a packet is one weight load, two (TSC) or
-                // one (CIC) 16/8-byte density loads and NQ/2 paired multiply-adds
-                auto qpairs = [&](const float *qp, f32x2 (&Q2)[NQ_ / 2]) {
-                    if constexpr (NQ_ == 8) {
-                        const ulonglong2 x = reinterpret_cast<const ulonglong2 *>(qp)[0];
-                        const ulonglong2 y = reinterpret_cast<const ulonglong2 *>(qp)[1];
-                        Q2[0] = x.x; Q2[1] = x.y; Q2[2] = y.x; Q2[3] = y.y;
-                    } else {
-                        Q2[0] = *reinterpret_cast<const f32x2 *>(qp);
-                    }
-                };
-                if (origin != carry_origin) {  // a new run: its first packet starts the sums
-                    flush_acc(carry_origin);
-                    carry_origin = origin;
-                    const f32x2 W2 = f2_pack(wrow[0], wrow[0]);
-                    f32x2 Q2[NQ_ / 2];
-                    qpairs(qrow, Q2);
+            if (origin != carry_origin) {  // a new run: its first packet starts the sums
+                flush_acc(carry_origin);
+                carry_origin = origin;
+                const T W = wrow[0];
+                T Qp[NQ_];
+                load_qpart<NQ_>(qrow, Qp);
 #pragma unroll
-                    for (int q = 0; q < NQ_ / 2; ++q)
-                        acc2[q] = f2_mul(W2, Q2[q]);
-                    ++p;
-                    wrow += WS;
-                    qrow += QO;
-                }
-                for (; p + 1 < R; p += 2, wrow += 2 * WS, qrow += 2 * QO) {
-                    const f32x2 Wa = f2_pack(wrow[0], wrow[0]), Wb = f2_pack(wrow[WS], wrow[WS]);
-                    f32x2 Qa[NQ_ / 2], Qb[NQ_ / 2];
-                    qpairs(qrow, Qa);
-                    qpairs(qrow + QO, Qb);
+                for (int q = 0; q < NQ_; ++q)
+                    acc[q] = W * Qp[q];
+                ++p;
+                wrow += WS;
+                qrow += QO;
+            }
+            for (; p + 1 < R; p += 2, wrow += 2 * WS, qrow += 2 * QO) {
+                const T W = wrow[0], W2 = wrow[WS];
+                T Qp[NQ_], Qp2[NQ_];
+                load_qpart<NQ_>(qrow, Qp);
+                load_qpart<NQ_>(qrow + QO, Qp2);
 #pragma unroll
-                    for (int q = 0; q < NQ_ / 2; ++q) {
-                        acc2[q] = f2_fma(Wa, Qa[q], acc2[q]);
-                        acc2[q] = f2_fma(Wb, Qb[q], acc2[q]);
-                    }
+                for (int q = 0; q < NQ_; ++q) {
+                    acc[q] += W * Qp[q];
+                    acc[q] += W2 * Qp2[q];
                 }
-                if (p < R) {
-                    const f32x2 W2 = f2_pack(wrow[0], wrow[0]);
-                    f32x2 Q2[NQ_ / 2];
-                    qpairs(qrow, Q2);
+            }
+            if (p < R) {
+                const T W = wrow[0];
+                T Qp[NQ_];
+                load_qpart<NQ_>(qrow, Qp);
 #pragma unroll
-                    for (int q = 0; q < NQ_ / 2; ++q)
-                        acc2[q] = f2_fma(W2, Q2[q], acc2[q]);
-                }
-            } else {
-                if (origin != carry_origin) {  // a new run: its first packet starts the sums
-                    flush_acc(carry_origin);
-                    carry_origin = origin;
-                    const T W = wrow[0];
-                    T Qp[NQ_];
-                    load_qpart<NQ_>(qrow, Qp);
-#pragma unroll
-                    for (int q = 0; q < NQ_; ++q)
-                        acc[q] = W * Qp[q];
-                    ++p;
-                    wrow += WS;
-                    qrow += QO;
-                }
-                for (; p + 1 < R; p += 2, wrow += 2 * WS, qrow += 2 * QO) {
-                    const T W = wrow[0], W2 = wrow[WS];
-                    T Qp[NQ_], Qp2[NQ_];
-                    load_qpart<NQ_>(qrow, Qp);
-                    load_qpart<NQ_>(qrow + QO, Qp2);
-#pragma unroll
-                    for (int q = 0; q < NQ_; ++q) {
-                        acc[q] += W * Qp[q];
-                        acc[q] += W2 * Qp2[q];
-                    }
-                }
-                if (p < R) {
-                    const T W = wrow[0];
-                    T Qp[NQ_];
-                    load_qpart<NQ_>(qrow, Qp);
-#pragma unroll
-                    for (int q = 0; q < NQ_; ++q)
-                        acc[q] += W * Qp[q];
-                }
+                for (int q = 0; q < NQ_; ++q)
+                    acc[q] += W * Qp[q];
             }
         }
         __syncwarp();
@@ -969,12 +677,12 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
     // add the deposit tile to the global grid (skip untouched nodes)
     for (int t = threadIdx.x; t < TE * TE * TE; t += blockDim.x) {
         const int lx = t % TE, ly = (t / TE) % TE, lz = t / (TE * TE);
-        const int slot = lz * DPS + ly * DRS + lx;
+        const int slot = lz * PS + ly * RS + lx;
         const int64_t node = s_axis[lx] + s_axis[TE + ly] + s_axis[2 * TE + lz];
         if (DET) {
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const long long v = sd[q * DTN + slot];
+                const long long v = sd[q * TN + slot];
                 if (v != 0)
                     atomicAdd(reinterpret_cast<unsigned long long *>(a.fx + node * 8 + q),
                               static_cast<unsigned long long>(v));
@@ -983,33 +691,487 @@ __device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, ui
             T v[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                v[q] = Cfg::I32 ? T(float(sd[q * DTN + slot]) * s_iscale[q]) : T(sd[q * DTN + slot]);
-            if (sizeof(T) == 4) {
-                float *p = reinterpret_cast<float *>(a.fb) + node * 8;
-                if (v[0] != T(0) || v[1] != T(0) || v[2] != T(0) || v[3] != T(0))
-                    atomicAdd(reinterpret_cast<float4 *>(p),
-                              make_float4(float(v[0]), float(v[1]), float(v[2]), float(v[3])));
-                if (v[4] != T(0) || v[5] != T(0) || v[6] != T(0) || v[7] != T(0))
-                    atomicAdd(reinterpret_cast<float4 *>(p + 4),
-                              make_float4(float(v[4]), float(v[5]), float(v[6]), float(v[7])));
-            } else {
+                v[q] = T(sd[q * TN + slot]);
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (v[q] != T(0))
-                        atomicAdd(reinterpret_cast<double *>(a.fb) + node * 8 + q, double(v[q]));
+            for (int q = 0; q < 8; ++q)
+                if (v[q] != T(0))
+                    atomicAdd(a.fb + node * 8 + q, v[q]);
+        }
+    }
+    if (flag)
+        atomicOr(a.status, flag);
+}
+
+
+// ---------------------------------------------------------------------------
+// FP32: packets pushed in memory order, deposited in octet order (octets.cuh).
+// ---------------------------------------------------------------------------
+template <int SHAPE, int B, int NW, bool DET>
+struct OctPushCfg {
+    // the deterministic deposit tile is twice as large, which leaves less to stage
+    using O = OctetCfg<SHAPE, B + 4, DET ? (B == 8 ? 1480 : 1024) : 2680, DET ? 16 : 32>;
+    static constexpr int TE = B + 4, TT = O::TT;
+    // deposit planes: 2 DTN = 8 mod 32 puts the four value pairs of a run on
+    // banks eight apart
+    static constexpr int DTN = TT + 4;
+    static_assert((2 * DTN) % 32 == 8, "deposit planes eight banks apart");
+    // Field tile as two planes, {Ex, Ey, Ez, Bx} and {By, Bz} per node, z planes two
+    // nodes apart: 16-byte loads of nearby nodes then spread over all banks.  (The
+    // lanes of a warp hold packets of four neighbouring cells when fresh, of
+    // about twenty after three steps of drift; with 32-byte nodes a gather load
+    // then took 10 wavefronts, here 5, and 3 when fresh.)
+    static constexpr int FZ = TE * TE + 2, FN = TE * FZ;
+    static constexpr size_t fields_bytes = size_t(FN) * 6 * sizeof(float);
+    // the bulk copy of the field tile (32-byte nodes) lands in the deposit tile
+    // (deterministic: 64-bit sums, low words in planes 0..7, high words in 8..15)
+    static constexpr size_t dep_bytes = size_t(DTN) * (DET ? 16 : 8) * sizeof(int);
+    static constexpr size_t raw_bytes = size_t(TT) * 8 * sizeof(float);
+    static_assert(raw_bytes <= dep_bytes && fields_bytes % 16 == 0, "field tile");
+    static constexpr size_t align_pad = 128;  // of the bulk copy's destination
+    static constexpr size_t smem_bytes = align_pad + dep_bytes + fields_bytes + O::stage_bytes + O::keep_bytes;
+};
+
+// One packet through global memory.  Not inlined: rare, and its unrolled gather
+// and deposit would take registers from the CTA body.
+template <int SHAPE, bool DET>
+__device__ __noinline__ int push_global(const PushArgs<float> &a, uint32_t j)
+{
+    int flag = 0;
+    auto gather_global = [&](int64_t node, float F[6]) { load_node(a.fields + node * 8, F); };
+    auto deposit_global = [&](int64_t node, float W, const float Q[8]) {
+        if constexpr (DET)
+            red_node_fixed(a.fx + node * 8, W, Q, a.fx_scale);
+        else
+            red_node(a.fb + node * 8, W, Q);
+    };
+    push_one<float, SHAPE, true>(a, int64_t(j), gather_global, deposit_global, &flag);
+    return flag;
+}
+
+// Add a 64-bit integer to the shared sum whose low word is *p and whose high word
+// lies HI words further, with native 32-bit atomics: the carry out of the low
+// word follows from the value the atomic returns.  (A 64-bit shared atomic is a
+// compare-and-swap loop.)  The order of the additions does not matter.
+template <int HI>
+__device__ __forceinline__ void add_fixed64(int *p, long long v)
+{
+    const uint32_t lo = uint32_t(v);
+    const uint32_t old = atomicAdd(reinterpret_cast<uint32_t *>(p), lo);
+    const int hi = int(v >> 32) + (old + lo < lo ? 1 : 0);
+    if (hi != 0)
+        atomicAdd(p + HI, hi);
+}
+
+// Parts of a bin of n packets: two chunks each.
+template <typename O>
+__device__ __forceinline__ uint32_t octet_parts(uint32_t n)
+{
+    return ((n + O::CHUNK - 1) / O::CHUNK + 1) / 2;
+}
+
+// Parts [part, part + n_parts) of the bin's packets [lo, hi).
+template <int SHAPE, int B, int NW, bool DET>
+__device__ __forceinline__ void octet_cta(const PushArgs<float> &a, uint32_t lo, uint32_t hi, int bx,
+                                          int by, int bz, uint32_t part, uint32_t n_parts,
+                                          const CUtensorMap *tmap = nullptr)
+{
+    using Cfg = OctPushCfg<SHAPE, B, NW, DET>;
+    using O = typename Cfg::O;
+    constexpr int TE = Cfg::TE, TT = Cfg::TT, DTN = Cfg::DTN, NP = O::NP, NS = O::NS, NT = NW * 32;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned char *smem = smem_raw + ((Cfg::align_pad - (smem_addr(smem_raw) & (Cfg::align_pad - 1))) &
+                                      (Cfg::align_pad - 1));
+    int *sd = reinterpret_cast<int *>(smem);  // first: 128-byte aligned
+    float4 *sf4 = reinterpret_cast<float4 *>(smem + Cfg::dep_bytes);
+    f32x2 *sf2 = reinterpret_cast<f32x2 *>(sf4 + Cfg::FN);
+    unsigned char *stage = smem + Cfg::dep_bytes + Cfg::fields_bytes;
+    const OctetMem<O> m(stage + O::stage_bytes, stage);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (lo >= hi)
+        return;
+    int flag = 0;
+    if (hi - lo <= sparse_cta_limit<SHAPE, B, DET>()) {
+        for (uint32_t j = lo + threadIdx.x; j < hi; j += NT)
+            flag |= push_global<SHAPE, DET>(a, j);
+        if (flag)
+            atomicOr(a.status, flag);
+        return;
+    }
+    const int ox = bx * B - 2, oy = by * B - 2, oz = bz * B - 2;
+    // A tile that does not wrap around the periodic grid on any axis is one box
+    // of the field grid: one bulk tensor copy (TMA) issued by thread 0 lands it
+    // while the threads count the origins below.
+    const bool tma = tmap != nullptr && ox >= 0 && oy >= 0 && oz >= 0 && ox + TE <= a.nx &&
+                     oy + TE <= a.ny && oz + TE <= a.nz;
+    __shared__ uint64_t s_tma_bar;
+    if (tma && threadIdx.x == 0)
+        mbar_init(&s_tma_bar, 1);
+    __shared__ int s_axis[3 * TE];
+    tile_axes<TE>(s_axis, ox, oy, oz, a.nx, a.ny, a.nz);
+    octet_clear<O, NW>(m);
+    __syncthreads();
+    if (tma && threadIdx.x == 0) {
+        mbar_arrive_expect_tx(&s_tma_bar, uint32_t(Cfg::raw_bytes));
+        tma_load_4d(sd, tmap, 0, ox, oy, oz, &s_tma_bar);
+    }
+    // a node of the tile into its planes; the fixed-point scale needs the largest
+    // |E| and, per axis a, the largest |B| across a (B with its a component removed)
+    float e2max = 0.f, bp2max[3] = {0.f, 0.f, 0.f};
+    auto set_node = [&](int t, const float F[6]) {
+        const int k = t + (t / (TE * TE)) * (Cfg::FZ - TE * TE);
+        sf4[k] = make_float4(F[0], F[1], F[2], F[3]);
+        sf2[k] = f2_pack(F[4], F[5]);
+        e2max = fmaxf(e2max, F[0] * F[0] + F[1] * F[1] + F[2] * F[2]);
+        const float bx2 = F[3] * F[3], by2 = F[4] * F[4], bz2 = F[5] * F[5];
+        bp2max[0] = fmaxf(bp2max[0], by2 + bz2);
+        bp2max[1] = fmaxf(bp2max[1], bx2 + bz2);
+        bp2max[2] = fmaxf(bp2max[2], bx2 + by2);
+    };
+    if (!tma) {
+        constexpr int UF = 4;  // nodes per thread per pass: all loads issued first
+        for (int t0 = threadIdx.x; t0 < TT; t0 += UF * NT) {
+            float F[UF][6];
+#pragma unroll
+            for (int u = 0; u < UF; ++u) {
+                const int t = t0 + u * NT;
+                if (t < TT) {
+                    const int node = s_axis[t % TE] + s_axis[TE + (t / TE) % TE] + s_axis[2 * TE + t / (TE * TE)];
+                    load_node(a.fields + int64_t(node) * 8, F[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < UF; ++u) {
+                const int t = t0 + u * NT;
+                if (t < TT)
+                    set_node(t, F[u]);
+            }
+        }
+    }
+    for (int t = threadIdx.x + (tma ? 2 * TT : 0); t < int(Cfg::dep_bytes / 16); t += NT)
+        reinterpret_cast<int4 *>(sd)[t] = make_int4(0, 0, 0, 0);
+
+    // Origin counts of packets [lo_, hi_), chunk 1 from packet split_ on, and each
+    // packet's origin and rank within it and its chunk; returns the largest |w|.
+    auto count_origins = [&](uint32_t lo_, uint32_t split_, uint32_t hi_) {
+        float wmax = 0.f;
+        constexpr int U = 4;  // packets per thread per pass: all loads issued first
+        for (uint32_t j0 = lo_ + threadIdx.x; j0 < hi_; j0 += U * NT) {
+            uint32_t cc[U];
+            float f0[U], f1[U], f2[U], ww[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t j = j0 + uint32_t(u) * NT;
+                const bool ok = j < hi_;
+                cc[u] = ok ? a.cell[j] : 0xFFFFFFFFu;
+                f0[u] = ok ? a.off0[j] : 0.f;
+                f1[u] = ok ? a.off1[j] : 0.f;
+                f2[u] = ok ? a.off2[j] : 0.f;
+                ww[u] = ok ? a.w[j] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t j = j0 + uint32_t(u) * NT;
+                wmax = fmaxf(wmax, fabsf(ww[u]));
+                // tile slot of the stencil's first node; out of the tile or off the grid: TT
+                const int ix = cell_x(cc[u]), iy = cell_y(cc[u]), iz = cell_z(cc[u]);
+                const int lx = wrap_once(ix + first_node<SHAPE>(f0[u]) - ox, a.nx),
+                          ly = wrap_once(iy + first_node<SHAPE>(f1[u]) - oy, a.ny),
+                          lz = wrap_once(iz + first_node<SHAPE>(f2[u]) - oz, a.nz);
+                const bool in = ix < a.nx && iy < a.ny && iz < a.nz && max(max(lx, ly), lz) <= TE - NP;
+                const int key = in ? (lz * TE + ly) * TE + lx : TT;
+                int *h = m.hist + (j >= split_ ? TT : 0) + key;
+                if (key < TT)
+                    m.rank[j - lo_] = uint16_t(atomicAdd(h, 1));
+                if (j < hi_)
+                    m.key[j - lo_] = uint16_t(key);
+            }
+        }
+        return wmax;
+    };
+    const int pair = lane & 3;
+    auto flush = [&](int slot, f32x2 (&acc)[NS]) {
+        int *p = sd + 2 * pair * DTN + slot;
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            const int off = (k / (NP * NP)) * TE * TE + ((k / NP) % NP) * TE + k % NP;
+            float x, y;
+            f2_unpack(acc[k], x, y);
+            if constexpr (DET) {
+                add_fixed64<8 * DTN>(p + off, to_fixed(x * a.fx_scale));
+                add_fixed64<8 * DTN>(p + DTN + off, to_fixed(y * a.fx_scale));
+            } else {  // values staged pre-scaled
+                atomicAdd(p + off, __float2int_rn(x));
+                atomicAdd(p + DTN + off, __float2int_rn(y));
+            }
+        }
+    };
+    // The bin in chunks of nearly equal size (all but the last a multiple of the CTA
+    // where that leaves room in the last), ordered two at a time.  Each two chunks
+    // have their own scale, from the packets in them, and their own tile.
+    const uint32_t n_bin = hi - lo, n_chunks = (n_bin + O::CHUNK - 1) / O::CHUNK;
+    uint32_t chunk = (n_bin + n_chunks - 1) / n_chunks;
+    if (chunk >= uint32_t(NT) && n_bin - chunk / NT * NT * (n_chunks - 1) <= O::CHUNK)
+        chunk = chunk / NT * NT;
+    const uint32_t c_first = 2 * part;
+    const uint32_t c_end = n_parts < octet_parts<O>(n_bin) - part ? 2 * (part + n_parts) : n_chunks;
+    __shared__ float s_scale[8], s_iscale[8];
+#pragma unroll 1
+    for (uint32_t c = c_first; c < c_end; c += 2) {
+        const uint32_t p_lo = lo + c * chunk;
+        const uint32_t split = c + 1 < n_chunks ? p_lo + chunk : hi;
+        const uint32_t p_hi = c + 2 < n_chunks ? split + chunk : hi;
+        if (c > c_first) {
+            __syncthreads();  // the previous part's tile has been added and cleared
+            octet_clear<O, NW>(m);
+            __syncthreads();
+        }
+        const float wmax = count_origins(p_lo, split, p_hi);
+        __syncthreads();
+        if constexpr (DET)
+            octet_stable_ranks<O, NW>(m, int(split - p_lo), int(p_hi - p_lo));
+        // the weight bound's three passes run between the order's barriers
+        float gmax = 0.f;
+        auto bound_pass = [&](int pass) {
+            if (!DET)
+                weight_bound_pass<SHAPE, TE, TE, TE * TE>(
+                    pass, [&](int t) { return m.hist[t] + m.hist[TT + t]; }, m.scratch, gmax);
+        };
+        int noct[2];
+        octet_order<O, NW>(m, int(split - p_lo), int(p_hi - p_lo), noct, bound_pass);
+        if (tma && c == c_first) {
+            // the bulk copy: wait for it (bounded), then the planes from the copied tile,
+            // which is cleared for the deposit
+            const bool arrived = mbar_wait_bounded(&s_tma_bar, 0, kTmaWaitCycles);
+            if (!__syncthreads_and(arrived)) {
+                // report it, give the copy one more bounded wait, skip the bin
+                if (threadIdx.x == 0) {
+                    atomicOr(a.status, ST_TIMEOUT);
+                    mbar_wait_bounded(&s_tma_bar, 0, kTmaWaitCycles);
+                }
+                __syncthreads();
+                return;
+            }
+            for (int t = threadIdx.x; t < TT; t += NT) {
+                float F[6];
+                lds_node(reinterpret_cast<const float *>(sd) + t * 8, F);
+                set_node(t, F);
+                reinterpret_cast<int4 *>(sd)[2 * t] = make_int4(0, 0, 0, 0);
+                reinterpret_cast<int4 *>(sd)[2 * t + 1] = make_int4(0, 0, 0, 0);
+            }
+        }
+        // 32-bit fixed point: scale_q = 2^e with (largest weight a node can receive) *
+        // bound_q below 2^31 / 1.002 (the margin covers the rounding of the bound and
+        // of the sums added), bound_q a bound on one packet's |Q_q| (|beta_bar| < 1):
+        //   rho: w q / dx^3;  J: rho c;  S_a: rho (|E| + |B across a|), since
+        //   |(beta_bar x B)_a| <= |beta_bar| |B with its a component removed|;
+        //   H: rho c |E| (1 + h |E|)
+        // (deterministic: the context's scale, in 64 bits)
+        if constexpr (!DET) {
+            __shared__ float s_red[6][NW];
+            float red[6] = {e2max, wmax, bp2max[0], bp2max[1], bp2max[2], gmax};
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int k = 0; k < 6; ++k)
+                    red[k] = fmaxf(red[k], __shfl_xor_sync(0xffffffffu, red[k], o));
+            if (lane == 0)
+#pragma unroll
+                for (int k = 0; k < 6; ++k)
+                    s_red[k][warp] = red[k];
+            __syncthreads();
+            if (threadIdx.x < 8) {
+                const int q = threadIdx.x;
+                const int bp = q >= 4 && q < 7 ? 2 + (q - 4) : 2;  // S_q: |B| across axis q - 4
+                float em = 0.f, bm = 0.f, wm = 0.f, gm = 0.f;
+                for (int w = 0; w < NW; ++w) {
+                    em = fmaxf(em, s_red[0][w]);
+                    wm = fmaxf(wm, s_red[1][w]);
+                    bm = fmaxf(bm, s_red[bp][w]);
+                    gm = fmaxf(gm, s_red[5][w]);
+                }
+                em = sqrtf(em);
+                bm = sqrtf(bm);
+                const float rho = wm * fabsf(a.k.qv);
+                float bound = q == 0 ? rho
+                            : q < 4  ? rho * a.k.c
+                            : q < 7  ? rho * (em + bm)
+                                     : rho * a.k.c * em * (1.f + fabsf(a.k.h) * em);
+                bound *= gm > 1.f ? gm : 1.f;
+                bound *= 1.002f;
+                int e = 30;
+                if (bound > 0.f && isfinite(bound))
+                    e = 31 - int(ceilf(log2f(bound)));
+                e = e > 60 ? 60 : (e < -60 ? -60 : e);
+                s_scale[q] = ldexpf(1.0f, e);
+                s_iscale[q] = ldexpf(1.0f, -e);
+            }
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int ch = 0; ch < 2; ++ch) {
+            const uint32_t c_lo = ch ? split : p_lo, c_hi = ch ? p_hi : split;
+            if (c_lo >= c_hi)
+                break;
+            // software pipeline: a thread's next packet is loaded into registers while
+            // this one is pushed
+            uint32_t n_c = 0;
+            int n_place = 0;
+            float n_o[3] = {0.f, 0.f, 0.f}, n_u[3] = {0.f, 0.f, 0.f}, n_w = 0.f;
+            auto prefetch = [&](uint32_t j) {
+                if (j < c_hi) {
+                    n_place = m.place[j - p_lo];
+                    n_c = a.cell[j];
+                    n_o[0] = a.off0[j];
+                    n_o[1] = a.off1[j];
+                    n_o[2] = a.off2[j];
+                    n_u[0] = a.u0[j];
+                    n_u[1] = a.u1[j];
+                    n_u[2] = a.u2[j];
+                    n_w = a.w[j];
+                }
+            };
+            prefetch(c_lo + threadIdx.x);
+            for (uint32_t j = c_lo + threadIdx.x; j < c_hi; j += NT) {
+                const uint32_t c = n_c;
+                const int place = n_place;
+                float fx = n_o[0], fy = n_o[1], fz = n_o[2];
+                const float u0[3] = {n_u[0], n_u[1], n_u[2]};
+                const float wj = n_w;
+                prefetch(j + NT);
+                const int ix = cell_x(c), iy = cell_y(c), iz = cell_z(c);
+                if (place == kOctNone) {  // off the grid, or drifted out of the tile since the sort
+                    flag |= push_global<SHAPE, DET>(a, j);
+                    continue;
+                }
+                float wx[3], wy[3], wz[3];
+                // tile slot of the stencil's first node (place is set: it lies in the tile)
+                const int slot = wrap_once(iz + axis_weights<SHAPE>(fz, wz) - oz, a.nz) * Cfg::FZ +
+                                 wrap_once(iy + axis_weights<SHAPE>(fy, wy) - oy, a.ny) * TE +
+                                 wrap_once(ix + axis_weights<SHAPE>(fx, wx) - ox, a.nx);
+                // pairs {Ex, Ey}, {Ez, Bx}, {By, Bz}: a node is one 16-byte and one
+                // 8-byte load, one paired product (its weight in both halves) and
+                // three paired multiply-adds; same bits as the order-free kernel
+                f32x2 g01 = 0, g23 = 0, g45 = 0;  // +0.0f in both halves
+                f32x2 wx2[NP];
+#pragma unroll
+                for (int cx = 0; cx < NP; ++cx)
+                    wx2[cx] = f2_pack(wx[cx], wx[cx]);
+                const float4 *p4 = sf4 + slot;
+                const f32x2 *p2 = sf2 + slot;
+#pragma unroll
+                for (int k = 0; k < NP * NP; ++k) {
+                    const float wyz = wy[k % NP] * wz[k / NP];
+                    const f32x2 wk = f2_pack(wyz, wyz);
+#pragma unroll
+                    for (int cx = 0; cx < NP; ++cx) {
+                        const f32x2 W2 = f2_mul(wx2[cx], wk);
+                        const int off = (k / NP) * Cfg::FZ + (k % NP) * TE + cx;
+                        const ulonglong2 a2 = *reinterpret_cast<const ulonglong2 *>(p4 + off);
+                        const f32x2 b2 = p2[off];
+                        g01 = f2_fma(W2, a2.x, g01);
+                        g23 = f2_fma(W2, a2.y, g23);
+                        g45 = f2_fma(W2, b2, g45);
+                    }
+                }
+                float E[3], Bf[3];
+                f2_unpack(g01, E[0], E[1]);
+                f2_unpack(g23, E[2], Bf[0]);
+                f2_unpack(g45, Bf[1], Bf[2]);
+                const BorisOut<float> b = boris(a.k.h, E, Bf, u0);
+                const float g0 = Math<float>::sqrt(1.f + dot3(u0, u0));
+                float Q[8];
+                feedback(a.k, wj, E, Bf, b, g0, Q);
+                if constexpr (!DET) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)  // the tile's fixed-point scale (a power of two: exact)
+                        Q[q] *= s_scale[q];
+                }
+                octet_stage<O>(m, place, octet_offset<SHAPE>(fx), octet_offset<SHAPE>(fy),
+                                       octet_offset<SHAPE>(fz), Q);
+                if (Math<float>::finite(b.u1[0]) && Math<float>::finite(b.u1[1]) &&
+                    Math<float>::finite(b.u1[2])) {
+                    const float s = a.k.adv * b.inv_g1;
+                    const int nx_ = drift_axis(ix, fx, s * b.u1[0], a.nx, &flag);
+                    const int ny_ = drift_axis(iy, fy, s * b.u1[1], a.ny, &flag);
+                    const int nz_ = drift_axis(iz, fz, s * b.u1[2], a.nz, &flag);
+                    a.cell[j] = pack_cell(nx_, ny_, nz_);
+                    a.off0[j] = fx;
+                    a.off1[j] = fy;
+                    a.off2[j] = fz;
+                    a.u0[j] = b.u1[0];
+                    a.u1[j] = b.u1[1];
+                    a.u2[j] = b.u1[2];
+                } else {
+                    flag |= ST_NONFINITE;
+                }
+            }
+            __syncthreads();
+            octet_deposit<O, NW, !DET>(m, ch, noct[ch], flush);
+            __syncthreads();  // the next chunk reuses the stage
+        }
+        // add the deposit tile to the global grid (skip untouched nodes); exact 64-bit
+        // sums wait for the last part
+        if (DET && c + 2 < c_end)
+            continue;
+        for (int t = threadIdx.x; t < TT; t += NT) {
+            const int64_t node = s_axis[t % TE] + s_axis[TE + (t / TE) % TE] + s_axis[2 * TE + t / (TE * TE)];
+            if constexpr (DET) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const unsigned long long v = uint32_t(sd[q * DTN + t]) |
+                                                 (unsigned long long)(uint32_t(sd[(8 + q) * DTN + t])) << 32;
+                    if (v != 0)
+                        atomicAdd(reinterpret_cast<unsigned long long *>(a.fx + node * 8 + q), v);
+                }
+            } else {
+                float v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    v[q] = float(sd[q * DTN + t]) * s_iscale[q];
+                    sd[q * DTN + t] = 0;
+                }
+                float *p = a.fb + node * 8;
+                if (v[0] != 0.f || v[1] != 0.f || v[2] != 0.f || v[3] != 0.f)
+                    atomicAdd(reinterpret_cast<float4 *>(p), make_float4(v[0], v[1], v[2], v[3]));
+                if (v[4] != 0.f || v[5] != 0.f || v[6] != 0.f || v[7] != 0.f)
+                    atomicAdd(reinterpret_cast<float4 *>(p + 4), make_float4(v[4], v[5], v[6], v[7]));
             }
         }
     }
     if (flag)
         atomicOr(a.status, flag);
-    if (tma && threadIdx.x == 0)  // every thread waited on it before the batches
+    if (tma && threadIdx.x == 0)  // every thread waited on it before the chunks
         mbar_inval(&s_tma_bar);
+}
+
+// The CTA body and its shared memory: octet order for FP32, one run per pass for FP64
+// (whose accumulators, a double per node and value, would not fit the registers).
+template <typename T>
+constexpr bool kUsesOctets = sizeof(T) == 4;
+template <typename T, int SHAPE, int B, int NW, bool DET>
+constexpr size_t tile_smem_bytes()
+{
+    if constexpr (kUsesOctets<T>)
+        return OctPushCfg<SHAPE, B, NW, DET>::smem_bytes;
+    else
+        return BinnedCfg<T, SHAPE, B, NW, DET>::smem_bytes;
+}
+template <typename T, int SHAPE, int B, int NW, bool DET>
+__device__ __forceinline__ void tile_cta(const PushArgs<T> &a, uint32_t lo, uint32_t hi, int bx, int by,
+                                         int bz, uint32_t part = 0, uint32_t n_parts = 0xFFFFFFFFu,
+                                         const CUtensorMap *tmap = nullptr)
+{
+    if constexpr (kUsesOctets<T>)
+        octet_cta<SHAPE, B, NW, DET>(a, lo, hi, bx, by, bz, part, n_parts, tmap);
+    else
+        binned_cta<T, SHAPE, B, NW, DET>(a, lo, hi, bx, by, bz);
 }
 
 template <typename T, int SHAPE, int B, int NW, bool DET>
 __global__ void __launch_bounds__(NW * 32)
-    push_binned_kernel(PushArgs<T> a, BinGeom g, int ahead, const __grid_constant__ CUtensorMap tmap,
-                       int use_tma)
+    push_binned_kernel(const __grid_constant__ PushArgs<T> a, const __grid_constant__ BinGeom g,
+                       int ahead, const __grid_constant__ CUtensorMap tmap, int use_tma)
 {
     const int bin = blockIdx.x;
     const int bx = bin % g.nbx, by = (bin / g.nbx) % g.nby, bz = bin / (g.nbx * g.nby);
@@ -1025,8 +1187,8 @@ __global__ void __launch_bounds__(NW * 32)
         prefetch_l2(a.u2, plo, phi);
         prefetch_l2(a.w, plo, phi);
     }
-    binned_cta<T, SHAPE, B, NW, DET>(a, g.bin_start[bin], g.bin_start[bin + 1], bx, by, bz,
-                                     use_tma ? &tmap : nullptr);
+    tile_cta<T, SHAPE, B, NW, DET>(a, g.bin_start[bin], g.bin_start[bin + 1], bx, by, bz,
+                                   0, 0xFFFFFFFFu, use_tma ? &tmap : nullptr);
 }
 
 // One box of a batch: grid, node offset into the concatenated grids, first
@@ -1071,12 +1233,12 @@ __device__ __forceinline__ PushArgs<T> batch_box_args(const PushArgs<T> &base, c
     return a;
 }
 
-// Work area of a batch push (device, 3 + total_bins words): claim counters,
+// Work area of a batch push (device, batch_work_words): claim counters,
 // zeroed before each push, and the list of the dense bins of this push.
 constexpr int kClaimSparse = 0;  // next bin a warp of the sparse kernel claims
-constexpr int kDenseCount = 1;   // dense bins listed by the sparse kernel
+constexpr int kDenseCount = 1;   // parts of dense bins listed by the sparse kernel
 constexpr int kClaimDense = 2;   // next list entry a CTA of the tiled kernel claims
-constexpr int kDenseList = 3;    // the list itself (at most total_bins entries)
+constexpr int kDenseList = 3;    // the list itself, a bin and a part each
 
 // The sparse bins of a batch (at most sparse_bin_limit packets): one warp per
 // bin, each lane one packet at a time, gathering from global memory and
@@ -1085,8 +1247,9 @@ constexpr int kDenseList = 3;    // the list itself (at most total_bins entries)
 // would stall a whole CTA on each sparse bin.  Warps claim the bins in order
 // from a counter (a bin's cost follows its packet count, so a fixed share per
 // warp would leave some warps with several large bins); a dense bin is only
-// listed for the tiled kernel.  Each bin is claimed once, so the list holds at
-// most total_bins entries.
+// listed for the tiled kernel, an entry per part.  Each bin is claimed once and a
+// bin of n packets has at most 1 + n / (2 chunk) parts, chunk >= 776, so the list
+// holds at most one entry per bin and one per 1024 packets.
 constexpr int kSparseWarps = 4;
 template <typename T, int SHAPE, int B, bool DET>
 __global__ void __launch_bounds__(kSparseWarps * 32) push_batch_sparse_kernel(
@@ -1103,9 +1266,18 @@ __global__ void __launch_bounds__(kSparseWarps * 32) push_batch_sparse_kernel(
         if (lane == 0)  // the next claim is in flight while this bin is pushed
             next = atomicAdd(&work[kClaimSparse], 1u);
         const uint32_t lo = bin_start[gb], hi = bin_start[gb + 1];
-        if (hi - lo > sparse_bin_limit<B>()) {
-            if (lane == 0)
-                work[kDenseList + atomicAdd(&work[kDenseCount], 1u)] = gb;
+        if (hi - lo > sparse_bin_limit<T, B, DET>()) {
+            if (lane == 0) {
+                // one entry per part of the bin, so that a very dense bin is shared out
+                uint32_t parts = 1;
+                if constexpr (kUsesOctets<T>)
+                    parts = octet_parts<typename OctPushCfg<SHAPE, B, 16, DET>::O>(hi - lo);
+                const uint32_t at = atomicAdd(&work[kDenseCount], parts);
+                for (uint32_t p = 0; p < parts; ++p) {
+                    work[kDenseList + 2 * (at + p)] = gb;
+                    work[kDenseList + 2 * (at + p) + 1] = p;
+                }
+            }
         } else if (lo < hi) {
             const PushArgs<T> a = batch_box_args(base, boxes[batch_box_of(boxes, n_boxes, gb)]);
             auto gather_global = [&](int64_t node, T F[6]) { load_node(a.fields + node * 8, F); };
@@ -1125,9 +1297,8 @@ __global__ void __launch_bounds__(kSparseWarps * 32) push_batch_sparse_kernel(
 }
 
 // Persistent kernel over the dense bins the sparse kernel listed: CTAs claim
-// list entries from a counter (dynamic balance: a dense bin holds from just
-// over sparse_bin_limit to tens of thousands of packets); each bin is processed by the same
-// CTA body as the single-box kernel, with its box's geometry, grids and
+// list entries from a counter (dynamic balance: an entry holds from just over
+// sparse_bin_limit to 4352 packets); each is processed by the same CTA body as the single-box kernel, with its box's geometry, grids and
 // constants.
 template <typename T, int SHAPE, int B, int NW, bool DET>
 __global__ void __launch_bounds__(NW * 32) push_batch_kernel(PushArgs<T> base,
@@ -1136,12 +1307,13 @@ __global__ void __launch_bounds__(NW * 32) push_batch_kernel(PushArgs<T> base,
                                                              const uint32_t *__restrict__ bin_start,
                                                              uint32_t *work)
 {
-    __shared__ uint32_t s_gb;
+    __shared__ uint32_t s_gb, s_part;
     const uint32_t n_dense = work[kDenseCount];  // complete: the sparse kernel ran before
     for (;;) {
         if (threadIdx.x == 0) {
             const uint32_t i = atomicAdd(&work[kClaimDense], 1u);
-            s_gb = i < n_dense ? work[kDenseList + i] : 0xFFFFFFFFu;
+            s_gb = i < n_dense ? work[kDenseList + 2 * i] : 0xFFFFFFFFu;
+            s_part = i < n_dense ? work[kDenseList + 2 * i + 1] : 0u;
         }
         __syncthreads();
         const uint32_t gb = s_gb;
@@ -1152,7 +1324,7 @@ __global__ void __launch_bounds__(NW * 32) push_batch_kernel(PushArgs<T> base,
         PushArgs<T> a = batch_box_args(base, bx_);
         const int lb = int(gb - bx_.bin_base);
         const int bx = lb % bx_.nbx, by = (lb / bx_.nbx) % bx_.nby, bz = lb / (bx_.nbx * bx_.nby);
-        binned_cta<T, SHAPE, B, NW, DET>(a, bin_start[gb], bin_start[gb + 1], bx, by, bz);
+        tile_cta<T, SHAPE, B, NW, DET>(a, bin_start[gb], bin_start[gb + 1], bx, by, bz, s_part, 1);
         __syncthreads();  // the next bin reuses the shared tiles and s_gb
     }
 }
@@ -1162,9 +1334,11 @@ __global__ void __launch_bounds__(NW * 32) push_batch_kernel(PushArgs<T> base,
 template <typename T, int SHAPE, int B, bool DET>
 constexpr int binned_warps()
 {
+    if constexpr (kUsesOctets<T>)
+        return 16;
     using C0 = BinnedCfg<T, SHAPE, B, 0, DET>;
     constexpr size_t budget = 232448 - 1024;  // leave room for static shared memory
-    constexpr size_t fixed = C0::align_pad + C0::fields_bytes + C0::dep_bytes + C0::key_bytes;
+    constexpr size_t fixed = C0::fields_bytes + C0::dep_bytes;
     constexpr size_t per_warp = C0::stage_words * sizeof(T);
     constexpr size_t fit = fixed >= budget ? 0 : (budget - fixed) / per_warp;
     constexpr int cap = DET ? 8 : 16;  // deterministic kernels need more registers
@@ -1206,22 +1380,22 @@ template <typename T, int SHAPE, int B, bool DET, int NW>
 cudaError_t launch_binned_nw(const PushArgs<T> &a, const BinGeom &g, int nbins, int sm_count,
                              cudaStream_t s)
 {
-    using Cfg = BinnedCfg<T, SHAPE, B, NW, DET>;
-    static_assert(Cfg::smem_bytes <= 232448, "binned tile exceeds shared memory");
+    constexpr size_t smem = tile_smem_bytes<T, SHAPE, B, NW, DET>();
+    static_assert(smem <= 232448, "binned tile exceeds shared memory");
     auto kern = push_binned_kernel<T, SHAPE, B, NW, DET>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(Cfg::smem_bytes));
+                                         int(smem));
     if (e != cudaSuccess)
         return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, Cfg::smem_bytes);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);
     if (e != cudaSuccess)
         return e;
     const int wave = sm_count * (per_sm > 0 ? per_sm : 1);  // CTAs resident at a time
     // FP32 tiles: interior bins take their fields with one bulk tensor copy
     CUtensorMap map{};
-    const int use_tma = Cfg::I32 && encode_field_tile_map(&map, a.fields, a.nx, a.ny, a.nz, Cfg::TE);
-    kern<<<nbins, NW * 32, Cfg::smem_bytes, s>>>(a, g, wave, map, use_tma);
+    const int use_tma = sizeof(T) == 4 && encode_field_tile_map(&map, a.fields, a.nx, a.ny, a.nz, B + 4);
+    kern<<<nbins, NW * 32, smem, s>>>(a, g, wave, map, use_tma);
     return cudaGetLastError();
 }
 
@@ -1272,19 +1446,17 @@ cudaError_t launch_batch(const PushArgs<T> &a, const BatchBox<T> *boxes, int n_b
     if constexpr (NW < 4) {
         return cudaErrorInvalidConfiguration;
     } else {
-        using Cfg = BinnedCfg<T, SHAPE, B, NW, DET>;
+        constexpr size_t smem = tile_smem_bytes<T, SHAPE, B, NW, DET>();
         auto kern = push_batch_kernel<T, SHAPE, B, NW, DET>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(Cfg::smem_bytes));
+                                             int(smem));
         if (e != cudaSuccess)
             return e;
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, Cfg::smem_bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);
         if (e != cudaSuccess)
             return e;
         uint32_t grid = uint32_t(sm_count) * uint32_t(per_sm > 0 ? per_sm : 1);
-        if (grid > total_bins)
-            grid = total_bins > 0 ? total_bins : 1;
         // the sparse bins first (one warp per bin; the dense ones listed), then the
         // dense ones
         e = cudaMemsetAsync(work, 0, kDenseList * sizeof(uint32_t), s);
@@ -1300,7 +1472,7 @@ cudaError_t launch_batch(const PushArgs<T> &a, const BatchBox<T> *boxes, int n_b
         if (sgrid > sgrid_max)
             sgrid = sgrid_max > 0 ? sgrid_max : 1;
         sk<<<unsigned(sgrid), kSparseWarps * 32, 0, s>>>(a, boxes, n_boxes, bin_start, total_bins, work);
-        kern<<<grid, NW * 32, Cfg::smem_bytes, s>>>(a, boxes, n_boxes, bin_start, work);
+        kern<<<grid, NW * 32, smem, s>>>(a, boxes, n_boxes, bin_start, work);
         return cudaGetLastError();
     }
 }

@@ -283,7 +283,6 @@ rsol_status rsol_sort_push_subcycled(rsol_ctx *ctx, const rsol_particles *in, rs
     b.nbz = ctx->nbz;
     b.tile_mode = 1;
     b.warps = ctx->p.warps;
-    b.perm = ss.keys[0];  // free once the level sort has gathered the packets
     // sub-step s of the finest level: level k moves when s is a multiple of
     // 2^(top - k), i.e. the levels top .. top - ctz(s) (all at s = 0).  Each
     // moving level is one binned push over its own bins, with h, adv and the
