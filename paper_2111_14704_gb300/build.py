@@ -1,9 +1,7 @@
 """Build librsol.so in-tree with nvcc for sm_103a (GB300).
 
 Every translation unit compiles in parallel to an object file under
-``paper_2111_14704_gb300/_build/``; the FP64 kernels are compiled with
-``-fmad=false`` so every product is rounded as written.  Usage:
-``python -m paper_2111_14704_gb300.build`` or ``build()`` from Python.
+``paper_2111_14704_gb300/_build/``.  Usage: ``python -m paper_2111_14704_gb300.build`` or ``build()`` from Python.
 """
 from __future__ import annotations
 
@@ -25,16 +23,16 @@ COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", CSRC, "
 UNITS = {
     "rsol_api.cu": [],
     "push_f32.cu": [],
-    "push_f64.cu": ["-fmad=false"],
+    "push_f64.cu": [],
     "sort.cu": [],
     "sort_static.cu": [],
     "fields.cu": [],
     "batch.cu": [],
     "adjoint_f32.cu": [],
-    "adjoint_f64.cu": ["-fmad=false"],
+    "adjoint_f64.cu": [],
     "rsol_grad.cu": [],
     "subcycle_f32.cu": [],
-    "subcycle_f64.cu": ["-fmad=false"],
+    "subcycle_f64.cu": [],
     "rsol_subcycle.cu": [],
 }
 

@@ -1,5 +1,4 @@
-// Reverse-mode step (FP64), compiled with -fmad=false like the FP64 forward
-// step so that the recomputed forward quantities round as written.
+// Reverse-mode step (FP64).
 #include "adjoint_binned.cuh"
 
 namespace rsol {

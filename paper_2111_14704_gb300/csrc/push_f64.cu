@@ -1,5 +1,7 @@
-// FP64 instantiation of the push, state-moment and totals kernels.  Compiled
-// with -fmad=false so every product is rounded as written (like the oracle).
+// FP64 instantiation of the push, state-moment and totals kernels.  Fused
+// multiply-adds are allowed: the FP64 pipe (two lanes a clock and SM) bounds these
+// kernels, and a fused operation rounds once instead of twice (2^21 packets on
+// 64^3 nodes, TSC: mean of four steps 4.93 -> 3.44 ms; 2^18 on 32^3, CIC: 322 -> 238 us).
 #include "push.cuh"
 #include "push_binned.cuh"
 #include "moments_binned.cuh"

@@ -1,4 +1,4 @@
-// FP64 instantiation of the sub-cycled push (-fmad=false, as push_f64.cu).
+// FP64 instantiation of the sub-cycled push.
 #include "subcycle.cuh"
 
 namespace rsol {
