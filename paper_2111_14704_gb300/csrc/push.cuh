@@ -280,6 +280,37 @@ __device__ __forceinline__ bool sum2_safe(float x)
     return (x == 0.f) | ((a >= 0x1p-40f) & (a <= 0x1p60f));
 }
 
+__device__ __forceinline__ void sum_into(double &a, double b) { a += b; }
+__device__ __forceinline__ void sum_into(Sum2 &a, const Sum2 &b) { a.add(b.hi, b.lo); }
+__device__ __forceinline__ double shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ Sum2 shfl_xor(const Sum2 &a, int o)
+{
+    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+
+// The warp's sums of 16 values per lane, value lane / 2 to each lane: each exchange
+// halves the values a lane holds, so 16 additions per lane where a reduction of each
+// value takes 80 (in FP64 those alone kept an SM for about 40 us per call).
+template <typename S>
+__device__ __forceinline__ S warp_sums16(S (&s)[16])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16, half = 8; half >= 1; o >>= 1, half >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < half; ++k) {
+            const S send = up ? s[k] : s[k + half];
+            S keep = up ? s[k + half] : s[k];
+            sum_into(keep, shfl_xor(send, o));
+            s[k] = keep;
+        }
+    }
+    S other = shfl_xor(s[0], 1);
+    sum_into(s[0], other);
+    return s[0];
+}
+
 // FP64 totals, first level: block b reduces a fixed contiguous chunk of packets
 // (and of feedback nodes) in a fixed order into partials[16][blocks].  gamma and
 // beta are formed in the packets' own precision (exact inputs, one rounding
@@ -294,10 +325,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(con
                                                      int64_t n_nodes, double mc, double mc2,
                                                      double qc, double vol, double *partials)
 {
-    double acc[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q)
-        acc[q] = 0.0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double total = 0.0;  // of value lane / 2
     const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
     const int64_t lo = int64_t(blockIdx.x) * chunk;
     const int64_t hi = lo + chunk < n ? lo + chunk : n;
@@ -359,12 +388,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(con
             }
         done = __syncthreads_and(safe);
         if (done) {
-#pragma unroll
-            for (int q = 0; q < 16; ++q)
-                acc[q] = s[q].value() * (q == 0 ? 1.0 : q < 4 ? mc : q == 4 ? mc2 : q < 8 ? qc : vol);
+            const int q = lane >> 1;
+            total = warp_sums16(s).value() * (q == 0 ? 1.0 : q < 4 ? mc : q == 4 ? mc2 : q < 8 ? qc : vol);
         }
     }
     if (!done) {
+        double acc[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+            acc[q] = 0.0;
         for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x) {
             const T uf[3] = {u0[j], u1[j], u2[j]};
             const T gf = Math<T>::sqrt(T(1) + dot3(uf, uf));
@@ -385,17 +417,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(con
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
                     acc[8 + q] += double(fb[i * 8 + q]) * vol;
+        total = warp_sums16(acc);
     }
     __shared__ double red[8][16];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            acc[q] += __shfl_down_sync(0xffffffffu, acc[q], o);
-        if (lane == 0)
-            red[warp][q] = acc[q];
-    }
+    if (lane % 2 == 0)
+        red[warp][lane >> 1] = total;
     __syncthreads();
     if (threadIdx.x < 16) {
         double t = red[0][threadIdx.x];
@@ -406,10 +432,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(con
 }
 
 // Second level: a warp per total sums its partials in a fixed order.
-static __global__ void __launch_bounds__(512) totals_final_kernel(const double *__restrict__ partials,
+static __global__ void __launch_bounds__(32) totals_final_kernel(const double *__restrict__ partials,
                                                                   int blocks, double *__restrict__ out)
 {
-    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int lane = threadIdx.x, q = blockIdx.x;
     double t = 0.0;
 #pragma unroll 8
     for (int b = lane; b < blocks; b += 32)
@@ -582,14 +608,17 @@ cudaError_t moments_dispatch(const MomentsDesc &d, cudaStream_t s)
 template <typename T>
 cudaError_t totals_dispatch(const TotalsDesc &d, cudaStream_t s)
 {
-    totals_kernel<T><<<d.blocks, 256, 0, s>>>(
+    // at least 1024 packets or nodes to a block: fewer do not pay for its reduction
+    const int64_t most = d.fb && d.n_nodes > d.n ? d.n_nodes : d.n, work = most / 1024 + 1;
+    const int blocks = work < d.blocks ? int(work) : d.blocks;
+    totals_kernel<T><<<blocks, 256, 0, s>>>(
         static_cast<const T *>(d.u[0]), static_cast<const T *>(d.u[1]),
         static_cast<const T *>(d.u[2]), static_cast<const T *>(d.w), d.n,
         static_cast<const T *>(d.fb), d.n_nodes, d.mc, d.mc2, d.qc, d.vol, d.partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;
-    totals_final_kernel<<<1, 512, 0, s>>>(d.partials, d.blocks, d.out);
+    totals_final_kernel<<<16, 32, 0, s>>>(d.partials, blocks, d.out);
     return cudaGetLastError();
 }
 
