@@ -29,9 +29,11 @@ struct ModeCoef {
 constexpr int MAX_MODES = 256;
 
 // Mode table passed by value as a kernel parameter (no host staging buffer,
-// so the launch can be captured in a CUDA graph).
+// so the launch can be captured in a CUDA graph).  N: 16, 64 or MAX_MODES; the
+// 18 KB of all 256 modes cost a launch several us of host time.
+template <int N>
 struct ModeSet {
-    ModeCoef m[MAX_MODES];
+    ModeCoef m[N];
 };
 
 size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
@@ -40,8 +42,10 @@ size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 // entries (re, im) of axis x (nx), then y (ny), then z (nz).
 // When tabx_t is given, the x entries are also written mode-fastest:
 // tabx_t[(i * n_modes + m) * 2 + {0, 1}].
-template <typename T>
-__global__ void tables_kernel(const ModeSet modes, int n_modes, int nx, int ny, int nz,
+// Bound by the FP64 pipe of the SMs it runs on (two lanes a clock): blocks of one
+// warp spread the few entries over the chip.
+template <typename T, int N>
+__global__ void __launch_bounds__(32) tables_kernel(const __grid_constant__ ModeSet<N> modes, int n_modes, int nx, int ny, int nz,
                               T *__restrict__ coef, T *__restrict__ tab, T *__restrict__ tabx_t = nullptr)
 {
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n_modes; m += gridDim.x * blockDim.x)
@@ -55,23 +59,23 @@ __global__ void tables_kernel(const ModeSet modes, int n_modes, int nx, int ny, 
          t += int64_t(gridDim.x) * blockDim.x) {
         const int m = int(t / len);
         int i = int(t % len);
-        int axis = 0, N = nx;
+        int axis = 0, L = nx;
         if (i >= nx) {
             i -= nx;
             axis = 1;
-            N = ny;
+            L = ny;
             if (i >= ny) {
                 i -= ny;
                 axis = 2;
-                N = nz;
+                L = nz;
             }
         }
         const ModeCoef &mc = modes.m[m];
-        // exact integer phase reduction: turns = (n_a * i mod N) / N
-        long long r = (static_cast<long long>(mc.n[axis]) * i) % N;
+        // exact integer phase reduction: turns = (n_a * i mod L) / L, L <= 1024
+        int r = (mc.n[axis] % L) * i % L;
         if (r < 0)
-            r += N;
-        double ang = 2.0 * double(r) / double(N);  // in units of pi
+            r += L;
+        double ang = 2.0 * double(r) / double(L);  // in units of pi
         double s, c;
         sincospi(ang, &s, &c);
         if (axis == 0) {
@@ -485,7 +489,7 @@ namespace {
 // Host-side mode coefficients: integer wave numbers, A e, -sigma vA A e / B0 and
 // the time-dependent phase psi = phi - sigma k_x vA t reduced to [0, 2 pi).
 // Mode m goes to place at[m] (in order when null).
-void fill_modes(ModeSet &hm, const double *h_modes, const double *h_sigma, int n_modes, double t,
+void fill_modes(ModeSet<MAX_MODES> &hm, const double *h_modes, const double *h_sigma, int n_modes, double t,
                 double B0, double vA, double dx, int nx, const int *at = nullptr)
 {
     const double two_pi = 6.283185307179586476925286766559;
@@ -506,6 +510,34 @@ void fill_modes(ModeSet &hm, const double *h_modes, const double *h_sigma, int n
     }
 }
 
+template <typename T, int N>
+void launch_tables_n(const ModeSet<MAX_MODES> &hm, int n_modes, int nx, int ny, int nz, void *coef, void *tab,
+                     void *tabx_t, cudaStream_t s)
+{
+    const int64_t blocks = (int64_t(n_modes) * (nx + ny + nz) + 31) / 32;
+    auto go = [&](const ModeSet<N> &set) {
+        tables_kernel<T, N><<<unsigned(blocks > 0 ? blocks : 1), 32, 0, s>>>(
+            set, n_modes, nx, ny, nz, static_cast<T *>(coef), static_cast<T *>(tab), static_cast<T *>(tabx_t));
+    };
+    if constexpr (N == MAX_MODES) {
+        go(hm);
+    } else {
+        ModeSet<N> set;
+        for (int m = 0; m < N; ++m)
+            set.m[m] = m < n_modes ? hm.m[m] : ModeCoef{};
+        go(set);
+    }
+}
+
+template <typename T>
+void launch_tables(const ModeSet<MAX_MODES> &hm, int n_modes, int nx, int ny, int nz, void *coef, void *tab,
+                   void *tabx_t, cudaStream_t s)
+{
+    auto f = n_modes <= 16 ? launch_tables_n<T, 16> : (n_modes <= 64 ? launch_tables_n<T, 64>
+                                                                     : launch_tables_n<T, MAX_MODES>);
+    f(hm, n_modes, nx, ny, nz, coef, tab, tabx_t, s);
+}
+
 } // namespace
 
 size_t alfven_scratch_bytes(int nx, int ny, int nz, int n_modes)
@@ -521,7 +553,7 @@ cudaError_t alfven_fields(const double *h_modes, const double *h_sigma, int n_mo
 {
     if (n_modes < 0 || n_modes > MAX_MODES)
         return cudaErrorInvalidValue;
-    static thread_local ModeSet hm;
+    static thread_local ModeSet<MAX_MODES> hm;
     int at[MAX_MODES], n_plus = 0;
     bool has_x = false, unit = true;
     static thread_local SigmaSet sg;
@@ -542,13 +574,9 @@ cudaError_t alfven_fields(const double *h_modes, const double *h_sigma, int n_mo
     const size_t esz = precision == 32 ? sizeof(float) : sizeof(double);
     void *coef = scratch;
     void *tab = static_cast<char *>(scratch) + align_up(size_t(n_modes) * 6 * esz);
-    const int64_t entries = int64_t(n_modes) * (nx + ny + nz);
-    const int tb = int((entries + 255) / 256) > 0 ? int((entries + 255) / 256) : 1;
     const dim3 grid(1, ny, nz);
     if (precision == 32) {
-        tables_kernel<float><<<tb, 256, 0, s>>>(hm, n_modes, nx, ny, nz,
-                                                static_cast<float *>(coef),
-                                                static_cast<float *>(tab));
+        launch_tables<float>(hm, n_modes, nx, ny, nz, coef, tab, nullptr, s);
         const dim3 rows(1, unsigned((ny + AF_ROWS - 1) / AF_ROWS), unsigned(nz));
         const size_t smem = size_t(n_modes) * (sizeof(float4) + sizeof(float2) * (2 + AF_ROWS));
         alfven_rows_kernel<<<rows, 32 * AF_ROWS, smem, s>>>(
@@ -556,9 +584,7 @@ cudaError_t alfven_fields(const double *h_modes, const double *h_sigma, int n_mo
             nz, float(B0), float(u_gas[0]), float(u_gas[1]), float(u_gas[2]), float(1.0 / c),
             static_cast<float *>(fields));
     } else {
-        tables_kernel<double><<<tb, 256, 0, s>>>(hm, n_modes, nx, ny, nz,
-                                                 static_cast<double *>(coef),
-                                                 static_cast<double *>(tab));
+        launch_tables<double>(hm, n_modes, nx, ny, nz, coef, tab, nullptr, s);
         auto kern = !unit ? alfven_kernel<true, false> : has_x ? alfven_kernel<true, true> : alfven_kernel<false, true>;
         kern<<<grid, 128, 0, s>>>(static_cast<const double *>(coef), n_modes, n_plus,
                                   static_cast<const double *>(tab), nx, ny, nz, B0, vA / B0, u_gas[0],
@@ -585,7 +611,7 @@ cudaError_t alfven_adjoint(const double *h_modes, const double *h_sigma, int n_m
 {
     if (n_modes < 1 || n_modes > MAX_MODES)
         return cudaErrorInvalidValue;
-    static thread_local ModeSet hm;
+    static thread_local ModeSet<MAX_MODES> hm;
     fill_modes(hm, h_modes, h_sigma, n_modes, t, B0, vA, dx, nx);
     // d/dA coefficients: e_m and kk_m = -sigma_m vA / B0 (kernel parameter, so
     // that the call can be captured in a CUDA graph)
@@ -604,13 +630,10 @@ cudaError_t alfven_adjoint(const double *h_modes, const double *h_sigma, int n_m
     double *partials = reinterpret_cast<double *>(after + align_up(size_t(n_modes) * 4 * sizeof(double)));
     void *tabx_t = after + align_up(size_t(n_modes) * 4 * sizeof(double)) +
                    align_up(size_t(ny) * nz * n_modes * sizeof(double));
-    const int64_t entries = int64_t(n_modes) * (nx + ny + nz);
-    const int tb = int((entries + 255) / 256) > 0 ? int((entries + 255) / 256) : 1;
     const dim3 grid(1, ny, nz);
     if (precision == 32) {
         acoef_kernel<float><<<1, 256, 0, s>>>(ac, n_modes, static_cast<float *>(acoef));
-        tables_kernel<float><<<tb, 256, 0, s>>>(hm, n_modes, nx, ny, nz, static_cast<float *>(coef),
-                                                static_cast<float *>(tab), static_cast<float *>(tabx_t));
+        launch_tables<float>(hm, n_modes, nx, ny, nz, coef, tab, tabx_t, s);
         alfven_adjoint_kernel<float><<<grid, 128, 0, s>>>(
             static_cast<const float *>(coef), static_cast<const float *>(acoef), n_modes,
             static_cast<const float *>(tab), static_cast<const float *>(tabx_t), nx, ny, nz, float(B0), float(u_gas[0]), float(u_gas[1]),
@@ -618,8 +641,7 @@ cudaError_t alfven_adjoint(const double *h_modes, const double *h_sigma, int n_m
             partials);
     } else {
         acoef_kernel<double><<<1, 256, 0, s>>>(ac, n_modes, static_cast<double *>(acoef));
-        tables_kernel<double><<<tb, 256, 0, s>>>(hm, n_modes, nx, ny, nz, static_cast<double *>(coef),
-                                                 static_cast<double *>(tab), static_cast<double *>(tabx_t));
+        launch_tables<double>(hm, n_modes, nx, ny, nz, coef, tab, tabx_t, s);
         alfven_adjoint_kernel<double><<<grid, 128, 0, s>>>(
             static_cast<const double *>(coef), static_cast<const double *>(acoef), n_modes,
             static_cast<const double *>(tab), static_cast<const double *>(tabx_t), nx, ny, nz, B0, u_gas[0], u_gas[1], u_gas[2], 1.0 / c,
