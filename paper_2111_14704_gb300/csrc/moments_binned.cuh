@@ -684,9 +684,13 @@ struct LossBinArgs {
 // Catastrophic losses (Sec. 2) for the last sort's output with a gathered
 // n_n: one CTA per bin stages the bin's n_n tile (bin + 2-node halo) in shared
 // memory and gathers each packet's n_n from it; packets whose stencil left the
-// tile read the grid.  Same arithmetic as losses_kernel.
+// tile read the grid.  Same arithmetic as losses_kernel.  Bound by the latency of the
+// packets' loads and by issue: FP32 at 64 registers keeps four CTAs on an SM, with
+// three packets per thread in flight (2^24 packets, TSC: 164 -> 146 us; four packets at
+// 80 registers, three CTAs, was the former; two packets at 64 took 150 us, at 48
+// registers with spills 183 us).
 template <typename T, int SHAPE, int B>
-__global__ void __launch_bounds__(256) losses_binned_kernel(LossBinArgs<T> a)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) losses_binned_kernel(LossBinArgs<T> a)
 {
     constexpr int NP = SHAPE == 1 ? 2 : 3;
     constexpr int TE = B + 4;
@@ -713,13 +717,14 @@ __global__ void __launch_bounds__(256) losses_binned_kernel(LossBinArgs<T> a)
     }
     __syncthreads();
     int flag = 0;
-    constexpr int U = 4;  // packets per thread per pass: their loads are issued first
-    for (uint32_t jb = lo + threadIdx.x; jb < hi; jb += U * blockDim.x) {
+    constexpr uint32_t NT = 256;
+    constexpr int U = sizeof(T) == 4 ? 3 : 4;  // packets per thread per pass: their loads are issued first
+    for (uint32_t jb = lo + threadIdx.x; jb < hi; jb += U * NT) {
         uint32_t cc[U];
         T f0[U], f1[U], f2[U], v0[U], v1[U], v2[U], ww[U];
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-            const uint32_t j = jb + uint32_t(k) * blockDim.x;
+            const size_t j = size_t(jb) + k * NT;
             const bool ok = j < hi;
             cc[k] = ok ? a.cell[j] : 0xFFFFFFFFu;
             f0[k] = ok ? a.o0[j] : T(0);
@@ -732,7 +737,7 @@ __global__ void __launch_bounds__(256) losses_binned_kernel(LossBinArgs<T> a)
         }
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-            const uint32_t j = jb + uint32_t(k) * blockDim.x;
+            const size_t j = size_t(jb) + k * NT;
             if (j >= hi)
                 continue;
             const T u[3] = {v0[k], v1[k], v2[k]};
