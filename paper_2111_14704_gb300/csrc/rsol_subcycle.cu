@@ -285,7 +285,8 @@ rsol_status rsol_sort_push_subcycled(rsol_ctx *ctx, const rsol_particles *in, rs
     b.warps = ctx->p.warps;
     // sub-step s of the finest level: level k moves when s is a multiple of
     // 2^(top - k), i.e. the levels top .. top - ctz(s) (all at s = 0).  Each
-    // moving level is one binned push over its own bins, with h, adv and the
+    // moving level is one binned push over its own bins (or, where that is expected to
+    // be faster, one order-free push of its packets; FP32 only, the same packet bits), with h, adv and the
     // deposit scaled by 2^-k; the levels are disjoint packet sets sharing the
     // grids, so their launches commute.
     const long n_sub = 1L << top;
@@ -306,6 +307,19 @@ rsol_status rsol_sort_push_subcycled(rsol_ctx *ctx, const rsol_particles *in, rs
             dk.adv = adv * sc;
             dk.qv = qv * sc;
             dk.bin_start = ss.bin_start + int64_t(r0 + (top - k)) * nbins;
+            if (order_free_faster(ctx, count[k])) {  // few packets: the level's slice of the arrays
+                const int64_t at = starts[sd->max_level - k];
+                auto from = [&](const void *p) { return static_cast<char *>(const_cast<void *>(p)) + at * es; };
+                dk.n = count[k];
+                dk.cell += at;
+                for (int a = 0; a < 3; ++a) {
+                    dk.off[a] = from(dk.off[a]);
+                    dk.u[a] = from(dk.u[a]);
+                }
+                dk.w = from(dk.w);
+                dk.bin_start = nullptr;
+                dk.tile_mode = 0;
+            }
             e = ctx->p.precision == 32 ? rsol::push_f32(dk, cs) : rsol::push_f64(dk, cs);
             if (e != cudaSuccess)
                 return cuda_fail(ctx, e, "rsol_sort_push_subcycled: sub-step launch");
