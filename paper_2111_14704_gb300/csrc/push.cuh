@@ -316,7 +316,7 @@ __device__ __forceinline__ S warp_sums16(S (&s)[16])
 // beta are formed in the packets' own precision (exact inputs, one rounding
 // each), every product and sum in FP64; FP32 packets are summed with Sum2 on the
 // FP32 pipes instead (the FP64 pipe, two lanes a clock and SM, took 698 us for 2^24
-// packets, this takes 130 us at the same error against 64 bits), and a block that meets values
+// packets, this takes 93 us at the same error against 64 bits), and a block that meets values
 // outside Sum2's range starts over in FP64.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(const T *__restrict__ u0, const T *__restrict__ u1,
