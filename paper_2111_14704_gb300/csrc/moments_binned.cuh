@@ -438,8 +438,9 @@ __global__ void __launch_bounds__(512) moments_octet_kernel(const __grid_constan
             octet_clear<O, NW>(m);
             __syncthreads();
         }
-        // origin counts, origins and ranks; the largest weight and |u|^2
-        float wmax = 0.f, u2max = 0.f;
+        // origin counts, origins and ranks; the largest weight and |u|^2; a sum that is 0
+        // unless some packet's weight, |u|^2 or offset is not finite
+        float wmax = 0.f, u2max = 0.f, nonfinite = 0.f;
         constexpr int U = 4;  // packets per thread per pass: all loads issued first
         for (uint32_t j0 = p_lo + threadIdx.x; j0 < p_hi; j0 += U * NT) {
             uint32_t cc[U];
@@ -461,8 +462,10 @@ __global__ void __launch_bounds__(512) moments_octet_kernel(const __grid_constan
             for (int u = 0; u < U; ++u) {
                 const uint32_t j = j0 + uint32_t(u) * NT;
                 const float uu[3] = {v0[u], v1[u], v2[u]};
+                const float uu2 = dot3(uu, uu);
                 wmax = fmaxf(wmax, fabsf(ww[u]));
-                u2max = fmaxf(u2max, dot3(uu, uu));
+                u2max = fmaxf(u2max, uu2);
+                nonfinite = __fmaf_rn(0.f, ((f0[u] + f1[u]) + f2[u]) + (fabsf(ww[u]) + uu2), nonfinite);
                 const int ix = cell_x(cc[u]), iy = cell_y(cc[u]), iz = cell_z(cc[u]);
                 const int lx = wrap_once(ix + first_node<SHAPE>(f0[u]) - ox, a.nx),
                           ly = wrap_once(iy + first_node<SHAPE>(f1[u]) - oy, a.ny),
@@ -515,10 +518,14 @@ __global__ void __launch_bounds__(512) moments_octet_kernel(const __grid_constan
                                  : n1 * fabsf(a.qc);
             bound *= gm > 1.f ? gm : 1.f;
             bound *= 1.002f;
+            // a finite bound is at most 2^128, so e >= 22 - 128 and the values stay within
+            // what the rounding by addition holds; 2^120 leaves both scales normal numbers
             int e = top - 1;
             if (bound > 0.f && isfinite(bound))
                 e = top - int(ceilf(log2f(bound)));
-            e = e > 60 ? 60 : (e < -60 ? -60 : e);
+            e = e > 120 ? 120 : e;
+            if (!isfinite(bound))
+                nonfinite = bound;
             s_scale[threadIdx.x] = ldexpf(1.0f, e);
             s_iscale[threadIdx.x] = ldexpf(1.0f, -e);
             if (threadIdx.x == 0) {
@@ -530,7 +537,13 @@ __global__ void __launch_bounds__(512) moments_octet_kernel(const __grid_constan
                 s_ilo = ldexpf(1.0f, -k);
             }
         }
-        __syncthreads();
+        if (__syncthreads_or(nonfinite != 0.f)) {
+            // no bound for the integers (a value that is not finite, or sums that may
+            // leave the FP32 range): each packet to its own nodes, as in a sparse bin
+            for (uint32_t j = p_lo + threadIdx.x; j < p_hi; j += NT)
+                moments_global<SHAPE>(a, j);
+            continue;
+        }
 #pragma unroll 1
         for (int ch = 0; ch < 2; ++ch) {
             const uint32_t c_lo = ch ? split : p_lo, c_hi = ch ? p_hi : split;
