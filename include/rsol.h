@@ -117,9 +117,7 @@ const char *rsol_last_error(const rsol_ctx *ctx);
  * eight feedback densities into d_feedback when it is not NULL, drift x.
  * Updates parts->cell, off and u in place; w is read only.  dt > 0.  When
  * parts is the set the last rsol_sort wrote, the binned shared-memory kernel
- * runs; otherwise, and (FP32, params.warps = 0, not deterministic) where the
- * set is too small or too sparse for it to pay, a kernel that needs no ordering
- * runs (same results up to
+ * runs; otherwise a kernel that needs no ordering runs (same results up to
  * the order of floating-point additions; deterministic mode makes each of
  * them bitwise reproducible from run to run).  "The set the last rsol_sort
  * wrote" is decided by buffer identity: parts->cell and parts->n equal the

@@ -60,6 +60,19 @@ __host__ __device__ constexpr uint32_t sparse_cta_limit()
     return DET ? sparse_bin_limit<float, B, DET>() : B == 8 ? (SHAPE == 1 ? 384u : 160u) : 128u;
 }
 
+// Where a box has fewer bins than half the SMs, a sparse bin is dealt to `slices` CTAs
+// (bin_slices), which raises the crossover to `slices` times the limit: a CTA then waits
+// for 1 / slices of the bin's atomics (TSC, 512 packets a bin: 8 bins 16.6 -> 11.4 us per
+// push, 27 bins 16.8 -> 15.6).  At most 768 packets of an 8^3 bin (256 of a 4^3 one), 1.5
+// (4) a node on average, go through global FP32 sums, however idle the GPU is: those
+// round once per packet and node, a tile's integers once per run of packets.
+template <int SHAPE, int B, bool DET>
+__host__ __device__ constexpr uint32_t sliced_cta_limit(uint32_t slices)
+{
+    const uint32_t limit = sparse_cta_limit<SHAPE, B, DET>(), most = B == 8 ? 768u : 256u;
+    return DET ? limit : limit * slices < most ? limit * slices : most;
+}
+
 struct BinGeom {
     const uint32_t *bin_start;
     int nbx, nby, nbz;
@@ -1187,8 +1200,25 @@ __global__ void __launch_bounds__(NW * 32)
         prefetch_l2(a.u2, plo, phi);
         prefetch_l2(a.w, plo, phi);
     }
-    tile_cta<T, SHAPE, B, NW, DET>(a, g.bin_start[bin], g.bin_start[bin + 1], bx, by, bz,
-                                   0, 0xFFFFFFFFu, use_tma ? &tmap : nullptr);
+    const uint32_t lo = g.bin_start[bin], hi = g.bin_start[bin + 1];
+    if constexpr (kUsesOctets<T>) {
+        if (gridDim.y > 1) {  // a sparse bin in slices; a dense one is the first slice's
+            const uint32_t n = hi - lo, slice = blockIdx.y;
+            if (n <= sliced_cta_limit<SHAPE, B, DET>(gridDim.y)) {
+                const uint32_t share = (n + gridDim.y - 1) / gridDim.y;
+                const uint32_t s_hi = min((slice + 1) * share, n);
+                int flag = 0;
+                for (uint32_t i = slice * share + threadIdx.x; i < s_hi; i += NW * 32)
+                    flag |= push_global<SHAPE, DET>(a, lo + i);
+                if (flag)
+                    atomicOr(a.status, flag);
+                return;
+            }
+            if (slice > 0)
+                return;
+        }
+    }
+    tile_cta<T, SHAPE, B, NW, DET>(a, lo, hi, bx, by, bz, 0, 0xFFFFFFFFu, use_tma ? &tmap : nullptr);
 }
 
 // One box of a batch: grid, node offset into the concatenated grids, first
@@ -1395,7 +1425,8 @@ cudaError_t launch_binned_nw(const PushArgs<T> &a, const BinGeom &g, int nbins, 
     // FP32 tiles: interior bins take their fields with one bulk tensor copy
     CUtensorMap map{};
     const int use_tma = sizeof(T) == 4 && encode_field_tile_map(&map, a.fields, a.nx, a.ny, a.nz, B + 4);
-    kern<<<nbins, NW * 32, smem, s>>>(a, g, wave, map, use_tma);
+    const int slices = kUsesOctets<T> ? bin_slices(sm_count, nbins) : 1;
+    kern<<<dim3(unsigned(nbins), unsigned(slices)), NW * 32, smem, s>>>(a, g, wave, map, use_tma);
     return cudaGetLastError();
 }
 

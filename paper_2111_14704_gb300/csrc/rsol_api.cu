@@ -189,8 +189,7 @@ rsol_status rsol_push_gather(rsol_ctx *ctx, const rsol_particles *P, const void 
     d.nbx = ctx->nbx;
     d.nby = ctx->nby;
     d.nbz = ctx->nbz;
-    if (ctx->sorted_cell == P->cell && ctx->sorted_n == P->n &&
-        !(d_feedback && order_free_faster(ctx, P->n))) {
+    if (ctx->sorted_cell == P->cell && ctx->sorted_n == P->n) {
         d.bin_start = ctx->sort.bin_start;
         d.tile_mode = 1;
     }

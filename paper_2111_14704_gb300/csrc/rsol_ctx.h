@@ -71,26 +71,6 @@ inline rsol_status cuda_fail(rsol_ctx *ctx, cudaError_t e, const char *what)
     return fail(ctx, RSOL_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
-// Whether the order-free kernel is expected to beat the binned one on a sorted
-// FP32 set: where the packets are too few to fill the GPU with bins' CTAs, or the
-// bins too sparse for their tiles.  From one GB300, 8^3 bins, us per push:
-//   order-free  5 + n c          c = 0.36e-3 (TSC), 0.115e-3 (CIC)
-//   binned      a + b p per wave of CTAs, p = n / bins: a = 12, b = 7.8e-3 (TSC),
-//               a = 10, b = 4.7e-3 (CIC); below 512 packets a bin it has no tiles
-// (TSC, binned against order-free: 16^3 x 2^12 packets 37 / 11, 32^3 x 2^15 40 / 13,
-// 32^3 x 2^16 20.6 / 23, 64^3 x 2^18 121 / 81, 64^3 x 2^20 103 / 318.)  A caller who asks
-// for a CTA width asks for the binned kernel.
-inline bool order_free_faster(const rsol_ctx *ctx, int64_t n)
-{
-    if (ctx->p.precision != 32 || ctx->p.deterministic || ctx->bin != 8 || ctx->p.warps != 0)
-        return false;
-    const double p = double(n) / double(ctx->nbins);
-    const bool cic = ctx->p.shape == 1;
-    const double waves = double((ctx->nbins + ctx->sm_count - 1) / ctx->sm_count);
-    const double binned = waves * (cic ? 10.0 + 4.7e-3 * p : 12.0 + 7.8e-3 * p);
-    return 5.0 + double(n) * (cic ? 0.115e-3 : 0.36e-3) < binned;
-}
-
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 inline int elem_bytes(const rsol_ctx *ctx) { return ctx->p.precision == 32 ? 4 : 8; }

@@ -75,6 +75,12 @@ struct LossDesc {
 cudaError_t losses_f32(const LossDesc &d, cudaStream_t s);
 cudaError_t losses_f64(const LossDesc &d, cudaStream_t s);
 cudaError_t push_f32(const PushDesc &d, cudaStream_t s);
+// CTAs that a box of few bins deals a sparse bin to (FP32; at most one CTA per SM).
+inline int bin_slices(int sm_count, int64_t nbins)
+{
+    const int64_t spare = sm_count / nbins;
+    return spare < 1 ? 1 : spare > 16 ? 16 : int(spare);
+}
 // Batched push over the bins of many boxes (boxes: device array of BatchBox<T>;
 // work: device scratch of batch_work_words(total_bins, packets) words, overwritten).
 cudaError_t push_batch_f32(const PushDesc &d, const void *boxes, int n_boxes, uint32_t total_bins,

@@ -15,6 +15,57 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 constexpr int kMaxLevels = 16;
 
+// First packet of each level rank (and of the end) and the packets of its fullest bin,
+// one block per rank: out[0 .. levels], out[levels + 1 .. 2 levels].
+__global__ void __launch_bounds__(256) level_summary_kernel(const uint32_t *__restrict__ bin_start,
+                                                            int64_t nbins, int levels, uint32_t *out)
+{
+    __shared__ uint32_t s_most;
+    if (threadIdx.x == 0)
+        s_most = 0;
+    __syncthreads();
+    const uint32_t *start = bin_start + blockIdx.x * nbins;
+    uint32_t most = 0;
+    for (int64_t b = threadIdx.x; b < nbins; b += blockDim.x)
+        most = max(most, start[b + 1] - start[b]);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((threadIdx.x & 31) == 0)
+        atomicMax(&s_most, most);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        out[blockIdx.x] = start[0];
+        if (int(blockIdx.x) == levels - 1)
+            out[levels] = start[nbins];
+        out[levels + 1 + blockIdx.x] = s_most;
+    }
+}
+
+// Whether a FP32 level of n packets goes through the order-free kernel: only where no
+// bin holds more than the 768 packets that the binned kernel too sums in global FP32
+// (sliced_cta_limit), so that which kernel runs costs no accuracy, and only where it is
+// expected to be faster.  From one GB300, 8^3 bins, us per push, p packets per bin:
+//   order-free             max(12.5, 5 + 0.31e-3 n) TSC, max(5.2, 4 + 0.08e-3 n) CIC
+//   binned, per wave       10 + 0.07 p / slices TSC, 6.2 + 0.018 p / slices CIC in sparse
+//                          bins (160, 384 packets a slice); 11 + 9.5e-3 p, 10.5 + 3e-3 p in tiles
+// (binned / order-free, TSC: 16^3 nodes x 4096 packets 11.4 / 10.9, 40^3 x 16000 20.5 / 13.8,
+// 48^3 x 55296 26.8 / 23.4, 48^3 x 110592 32.2 / 41.4, 64^3 x 65536 71.5 / 24.2, x 262144
+// 63.3 / 80.5; CIC: 16^3 x 4096 6.2 / 4.9, 64^3 x 262144 47.2 / 24.8.)  A caller who asks
+// for a CTA width asks for the binned kernel.
+bool order_free_faster(const rsol_ctx *ctx, int64_t n, uint32_t fullest)
+{
+    if (ctx->p.precision != 32 || ctx->p.deterministic || ctx->bin != 8 || ctx->p.warps != 0 || fullest > 768)
+        return false;
+    const bool cic = ctx->p.shape == 1;
+    const double p = double(n) / double(ctx->nbins);
+    const int slices = rsol::bin_slices(ctx->sm_count, ctx->nbins);
+    const double waves = double((ctx->nbins + ctx->sm_count - 1) / ctx->sm_count);
+    const bool sparse = p <= double((cic ? 384 : 160) * slices);
+    const double binned = sparse ? (cic ? 6.2 + 0.018 * p / slices : 10.0 + 0.07 * p / slices)
+                                 : (cic ? 10.5 + 3e-3 * p : 11.0 + 9.5e-3 * p);
+    const double free = cic ? std::fmax(5.2, 4.0 + 0.08e-3 * n) : std::fmax(12.5, 5.0 + 0.31e-3 * n);
+    return free < waves * binned;
+}
+
 } // namespace
 
 extern "C" {
@@ -226,12 +277,17 @@ rsol_status rsol_sort_push_subcycled(rsol_ctx *ctx, const rsol_particles *in, rs
                                  out->w, lb, key_bits, nbins_total, cs);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "rsol_sort_push_subcycled: level sort");
-    ctx->launches += 2 + 4 * ((key_bits + 7) / 8);
+    ctx->launches += 3 + 4 * ((key_bits + 7) / 8);
 
-    // packets per level: the level ranks' first bins, read back once
-    uint32_t starts[kMaxLevels + 2];
-    e = cudaMemcpy2DAsync(starts, sizeof(uint32_t), ss.bin_start, size_t(nbins) * sizeof(uint32_t),
-                          sizeof(uint32_t), size_t(sd->max_level + 2), cudaMemcpyDeviceToHost, cs);
+    // packets per level and in its fullest bin, read back once (the sort is done with
+    // its block sums, 256 words)
+    const int levels = sd->max_level + 1;
+    uint32_t starts[2 * (kMaxLevels + 1) + 1];
+    const uint32_t *fullest = starts + levels + 1;
+    level_summary_kernel<<<levels, 256, 0, cs>>>(ss.bin_start, nbins, levels, ss.block_sums);
+    e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(starts, ss.block_sums, (2 * levels + 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost, cs);
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(cs);
     if (e != cudaSuccess)
@@ -285,8 +341,9 @@ rsol_status rsol_sort_push_subcycled(rsol_ctx *ctx, const rsol_particles *in, rs
     b.warps = ctx->p.warps;
     // sub-step s of the finest level: level k moves when s is a multiple of
     // 2^(top - k), i.e. the levels top .. top - ctz(s) (all at s = 0).  Each
-    // moving level is one binned push over its own bins (or, where that is expected to
-    // be faster, one order-free push of its packets; FP32 only, the same packet bits), with h, adv and the
+    // moving level is one binned push over its own bins (or, where its bins are sparse and
+    // that is expected to be faster, one order-free push of its packets; FP32 only, the same
+    // packet bits, sums of the same kind), with h, adv and the
     // deposit scaled by 2^-k; the levels are disjoint packet sets sharing the
     // grids, so their launches commute.
     const long n_sub = 1L << top;
@@ -307,7 +364,7 @@ rsol_status rsol_sort_push_subcycled(rsol_ctx *ctx, const rsol_particles *in, rs
             dk.adv = adv * sc;
             dk.qv = qv * sc;
             dk.bin_start = ss.bin_start + int64_t(r0 + (top - k)) * nbins;
-            if (order_free_faster(ctx, count[k])) {  // few packets: the level's slice of the arrays
+            if (order_free_faster(ctx, count[k], fullest[sd->max_level - k])) {  // the level's slice of the arrays
                 const int64_t at = starts[sd->max_level - k];
                 auto from = [&](const void *p) { return static_cast<char *>(const_cast<void *>(p)) + at * es; };
                 dk.n = count[k];
