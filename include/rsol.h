@@ -165,8 +165,9 @@ rsol_status rsol_sort(rsol_ctx *ctx, const rsol_particles *in, rsol_particles *o
  *   [5..7] sum N_j q c beta
  *   [8..15] sum over nodes of d_feedback's 8 components times dx^3
  *           (0 when d_feedback is NULL).
- * The reduction order is fixed, so repeated calls give identical bits.
- * Synchronises the stream.
+ * gamma and beta are formed in the context's precision; products and sums
+ * carry at least the 53 bits of FP64.  The reduction order is fixed, so
+ * repeated calls give identical bits.  Synchronises the stream.
  */
 rsol_status rsol_moments(rsol_ctx *ctx, const rsol_particles *parts,
                          const void *d_feedback, double *h_totals, void *stream);

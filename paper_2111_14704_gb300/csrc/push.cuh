@@ -253,50 +253,67 @@ __global__ void __launch_bounds__(256) moments_grid_kernel(MomArgs<T> a)
     }
 }
 
-// Sum of FP32 values held in two floats: every addition's rounding error is
-// recovered exactly (Knuth's two-sum) and summed beside it, so that the pair
-// carries about 48 bits.
-struct Sum2 {
-    float hi, lo;
-    __device__ __forceinline__ void add(float x, float rest = 0.f)
+// Sum of FP32 values held in three floats: the rounding error of every addition to hi
+// is recovered exactly (Knuth's two-sum) and added to mid, whose own errors are summed
+// in lo, so that the sum carries about 70 bits: more than FP64 terms and sums.
+struct Sum3 {
+    float hi, mid, lo;
+    // s + x into s; returns what the rounding lost (the intrinsics keep the compiler
+    // from fusing a product into the sum)
+    static __device__ __forceinline__ float two_sum(float &s, float x)
     {
-        // (the intrinsics keep the compiler from fusing a product into the sum)
-        const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
-        lo += __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b)), rest);
-        hi = t;
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+        s = t;
+        return e;
     }
+    __device__ __forceinline__ void add(float x) { lo = __fadd_rn(lo, two_sum(mid, two_sum(hi, x))); }
     __device__ __forceinline__ void add_product(float a, float x)  // exact: a x = p + fma(a, x, -p)
     {
         const float p = __fmul_rn(a, x);
-        add(p, __fmaf_rn(a, x, -p));
+        add(p);
+        lo = __fadd_rn(lo, two_sum(mid, __fmaf_rn(a, x, -p)));
     }
-    __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
+    __device__ __forceinline__ double value() const { return double(hi) + (double(mid) + double(lo)); }
 };
 
-// Whether Sum2 holds products of such values without overflow or a loss of low bits.
-__device__ __forceinline__ bool sum2_safe(float x)
+// Whether Sum3 is exact enough for a packet and cannot overflow: N, the weight scaled by
+// the block's power of two, in 2^-26 .. 2^26, and momenta in 2^-40 .. 2^33 (or 0).  The last
+// bit of the smallest product, N u / gamma, is then 2^(-26 - 23 - 40 - 34 - 23) = 2^-146, an
+// FP32 number, and 2^31 of the largest stay below 2^92.
+__device__ __forceinline__ bool sum3_weight(float x)
 {
     const float a = fabsf(x);
-    return (x == 0.f) | ((a >= 0x1p-40f) & (a <= 0x1p60f));
+    return (x == 0.f) | ((a >= 0x1p-26f) & (a <= 0x1p26f));
+}
+__device__ __forceinline__ bool sum3_momentum(float x)
+{
+    const float a = fabsf(x);
+    return (x == 0.f) | ((a >= 0x1p-40f) & (a <= 0x1p33f));
 }
 
 __device__ __forceinline__ void sum_into(double &a, double b) { a += b; }
-__device__ __forceinline__ void sum_into(Sum2 &a, const Sum2 &b) { a.add(b.hi, b.lo); }
-__device__ __forceinline__ double shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-__device__ __forceinline__ Sum2 shfl_xor(const Sum2 &a, int o)
+__device__ __forceinline__ void sum_into(Sum3 &a, const Sum3 &b)
 {
-    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+    a.add(b.hi);
+    a.lo = __fadd_rn(a.lo, __fadd_rn(Sum3::two_sum(a.mid, b.mid), b.lo));
+}
+__device__ __forceinline__ double shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ Sum3 shfl_xor(const Sum3 &a, int o)
+{
+    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.mid, o),
+            __shfl_xor_sync(0xffffffffu, a.lo, o)};
 }
 
-// The warp's sums of 16 values per lane, value lane / 2 to each lane: each exchange
-// halves the values a lane holds, so 16 additions per lane where a reduction of each
-// value takes 80 (in FP64 those alone kept an SM for about 40 us per call).
+// The warp's sums of 8 values per lane, value lane / 4 to each lane: each exchange
+// halves the values a lane holds, so 9 additions per lane where a reduction of each
+// value takes 40 (in FP64 those alone kept an SM for about 20 us per call).
 template <typename S>
-__device__ __forceinline__ S warp_sums16(S (&s)[16])
+__device__ __forceinline__ S warp_sums8(S (&s)[8])
 {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int o = 16, half = 8; half >= 1; o >>= 1, half >>= 1) {
+    for (int o = 16, half = 4; half >= 1; o >>= 1, half >>= 1) {
         const bool up = lane & o;
 #pragma unroll
         for (int k = 0; k < half; ++k) {
@@ -306,18 +323,22 @@ __device__ __forceinline__ S warp_sums16(S (&s)[16])
             s[k] = keep;
         }
     }
-    S other = shfl_xor(s[0], 1);
-    sum_into(s[0], other);
+#pragma unroll
+    for (int o = 2; o >= 1; o >>= 1) {
+        const S other = shfl_xor(s[0], o);
+        sum_into(s[0], other);
+    }
     return s[0];
 }
 
 // FP64 totals, first level: block b reduces a fixed contiguous chunk of packets
 // (and of feedback nodes) in a fixed order into partials[16][blocks].  gamma and
 // beta are formed in the packets' own precision (exact inputs, one rounding
-// each), every product and sum in FP64; FP32 packets are summed with Sum2 on the
-// FP32 pipes instead (the FP64 pipe, two lanes a clock and SM, took 698 us for 2^24
-// packets, this takes 93 us at the same error against 64 bits), and a block that meets values
-// outside Sum2's range starts over in FP64.
+// each), products and sums carry at least the 53 bits of FP64.  FP32 packets are summed
+// with Sum3, bound by the FP32 pipes; the FP64 pipe has two lanes a clock and SM (a call
+// for 2^24 packets: 155 us, 690 in FP64; 111 with sums of two floats, whose 48 bits
+// lost up to 226 2^-53 of a total where FP64 loses 6).  A block that meets values
+// outside Sum3's range sums in FP64, from its first 1024 packets on if they hold one.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(const T *__restrict__ u0, const T *__restrict__ u1,
                                                      const T *__restrict__ u2, const T *__restrict__ w,
@@ -325,8 +346,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(con
                                                      int64_t n_nodes, double mc, double mc2,
                                                      double qc, double vol, double *partials)
 {
+    constexpr int NT = 256;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double total = 0.0;  // of value lane / 2
+    double packets = 0.0, nodes = 0.0;  // of values lane / 4 and 8 + lane / 4
     const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
     const int64_t lo = int64_t(blockIdx.x) * chunk;
     const int64_t hi = lo + chunk < n ? lo + chunk : n;
@@ -335,17 +357,23 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(con
     const int64_t nhi = nlo + cn < n_nodes ? nlo + cn : n_nodes;
     bool done = false;
     if constexpr (sizeof(T) == 4) {
-        Sum2 s[16];
+        // weights by the power of two that takes the block's first one to 1 .. 2
+        int e = 0;
+        if (lo < hi && w[lo] != 0.f && isfinite(w[lo]))
+            e = ilogbf(w[lo]);
+        e = e > 100 ? 100 : (e < -100 ? -100 : e);
+        const float scale = ldexpf(1.f, -e);
+        Sum3 s[8];
 #pragma unroll
-        for (int q = 0; q < 16; ++q)
-            s[q] = {0.f, 0.f};
-        bool safe = true;
+        for (int q = 0; q < 8; ++q)
+            s[q] = {0.f, 0.f, 0.f};
+        bool safe = true, go = true;
         constexpr int U = 4;  // packets per thread per pass: all loads issued first
-        for (int64_t j0 = lo + threadIdx.x; j0 < hi; j0 += U * blockDim.x) {
+        for (int64_t base = lo; base < hi; base += U * NT) {  // block-uniform
             float N[U], v0[U], v1[U], v2[U];
 #pragma unroll
             for (int k = 0; k < U; ++k) {
-                const int64_t j = j0 + int64_t(k) * blockDim.x;
+                const int64_t j = base + threadIdx.x + k * NT;
                 const bool ok = j < hi;  // past the end: zeros, which add nothing
                 N[k] = ok ? w[j] : 0.f;
                 v0[k] = ok ? u0[j] : 0.f;
@@ -355,49 +383,56 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(con
 #pragma unroll
             for (int k = 0; k < U; ++k) {
                 const float uf[3] = {v0[k], v1[k], v2[k]};
+                const float m = __fmul_rn(N[k], scale);
                 const float gf = Math<float>::sqrt(1.f + dot3(uf, uf));
                 const float igf = 1.f / gf;
-                safe = safe & sum2_safe(N[k]) & sum2_safe(uf[0]) & sum2_safe(uf[1]) & sum2_safe(uf[2]);
-                s[0].add(N[k]);
-                s[4].add_product(N[k], gf);
+                safe = safe & sum3_weight(m) & sum3_momentum(uf[0]) & sum3_momentum(uf[1]) & sum3_momentum(uf[2]);
+                s[0].add(m);
+                s[4].add_product(m, gf);
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    s[1 + q].add_product(N[k], uf[q]);
-                    s[5 + q].add_product(N[k], uf[q] * igf);
+                    s[1 + q].add_product(m, uf[q]);
+                    s[5 + q].add_product(m, uf[q] * igf);
                 }
+            }
+            if (base == lo && !__syncthreads_and(safe)) {
+                go = false;
+                break;
             }
         }
-        const bool wide = (reinterpret_cast<uintptr_t>(fb) & 15) == 0;
-        if (fb)
-            for (int64_t i = nlo + threadIdx.x; i < nhi; i += blockDim.x) {
-                float v[8];
-                if (wide) {
-                    const float4 a = reinterpret_cast<const float4 *>(fb + i * 8)[0];
-                    const float4 b = reinterpret_cast<const float4 *>(fb + i * 8)[1];
-                    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-                } else {
+        if (go) {
+            const int q = lane >> 2;
+            packets = warp_sums8(s).value() * ldexp(q == 0 ? 1.0 : q < 4 ? mc : q == 4 ? mc2 : qc, e);
+            const bool wide = (reinterpret_cast<uintptr_t>(fb) & 15) == 0;
+            if (fb) {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        v[q] = fb[i * 8 + q];
-                }
+                for (int q = 0; q < 8; ++q)
+                    s[q] = {0.f, 0.f, 0.f};
+                for (int64_t i = nlo + threadIdx.x; i < nhi; i += NT) {
+                    float v[8];
+                    if (wide) {
+                        const float4 a = reinterpret_cast<const float4 *>(fb + i * 8)[0];
+                        const float4 b = reinterpret_cast<const float4 *>(fb + i * 8)[1];
+                        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+                    } else {
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    safe = safe & (fabsf(v[q]) <= 0x1p100f);
-                    s[8 + q].add(v[q]);
+                        for (int q = 0; q < 8; ++q)
+                            v[q] = fb[i * 8 + q];
+                    }
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        safe = safe & (fabsf(v[q]) <= 0x1p96f);  // at most 2^30 nodes
+                        s[q].add(v[q]);
+                    }
                 }
+                nodes = warp_sums8(s).value() * vol;
             }
-        done = __syncthreads_and(safe);
-        if (done) {
-            const int q = lane >> 1;
-            total = warp_sums16(s).value() * (q == 0 ? 1.0 : q < 4 ? mc : q == 4 ? mc2 : q < 8 ? qc : vol);
+            done = __syncthreads_and(safe);
         }
     }
     if (!done) {
-        double acc[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-            acc[q] = 0.0;
-        for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x) {
+        double acc[8] = {};
+        for (int64_t j = lo + threadIdx.x; j < hi; j += NT) {
             const T uf[3] = {u0[j], u1[j], u2[j]};
             const T gf = Math<T>::sqrt(T(1) + dot3(uf, uf));
             const T igf = T(1) / gf;
@@ -412,16 +447,24 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) totals_kernel(con
             for (int q = 0; q < 3; ++q)
                 acc[5 + q] += Nqc * double(uf[q] * igf);
         }
-        if (fb)
-            for (int64_t i = nlo + threadIdx.x; i < nhi; i += blockDim.x)
+        packets = warp_sums8(acc);
+        nodes = 0.0;
+        if (fb) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                acc[q] = 0.0;
+            for (int64_t i = nlo + threadIdx.x; i < nhi; i += NT)
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
-                    acc[8 + q] += double(fb[i * 8 + q]) * vol;
-        total = warp_sums16(acc);
+                    acc[q] += double(fb[i * 8 + q]) * vol;
+            nodes = warp_sums8(acc);
+        }
     }
     __shared__ double red[8][16];
-    if (lane % 2 == 0)
-        red[warp][lane >> 1] = total;
+    if (lane % 4 == 0) {
+        red[warp][lane >> 2] = packets;
+        red[warp][8 + (lane >> 2)] = nodes;
+    }
     __syncthreads();
     if (threadIdx.x < 16) {
         double t = red[0][threadIdx.x];
