@@ -75,7 +75,9 @@ typedef struct rsol_params {
     int32_t warps;         /* CTA width of the binned push, in warps: 8 or 16; 0 =     */
                            /* the widest that fits shared memory (16 for FP32).  The   */
                            /* Python package's autotuner picks bin and warps per GPU   */
-                           /* and workload; results do not depend on either.           */
+                           /* and workload.  Either changes the deposits only by the   */
+                           /* rounding of sums; with deterministic = 1 no bit depends  */
+                           /* on warps.                                                */
     double dx;             /* cell size (> 0)                                          */
     double c;              /* true speed of light (> 0)                                */
     double c_tilde;        /* reduced speed of light, 0 < c~ <= c                      */

@@ -919,13 +919,16 @@ __device__ __forceinline__ void octet_cta(const PushArgs<float> &a, uint32_t lo,
             }
         }
     };
-    // The bin in chunks of nearly equal size (all but the last a multiple of the CTA
-    // where that leaves room in the last), ordered two at a time.  Each two chunks
-    // have their own scale, from the packets in them, and their own tile.
+    // The bin in chunks of nearly equal size (all but the last a multiple of the widest
+    // CTA where that leaves room in the last), ordered two at a time.  Each two chunks
+    // have their own scale, from the packets in them, and their own tile.  The cut does
+    // not depend on this CTA's width: deterministic sums round per run, and the runs
+    // end with their chunk.
+    constexpr uint32_t STEP = 512;
     const uint32_t n_bin = hi - lo, n_chunks = (n_bin + O::CHUNK - 1) / O::CHUNK;
     uint32_t chunk = (n_bin + n_chunks - 1) / n_chunks;
-    if (chunk >= uint32_t(NT) && n_bin - chunk / NT * NT * (n_chunks - 1) <= O::CHUNK)
-        chunk = chunk / NT * NT;
+    if (chunk >= STEP && n_bin - chunk / STEP * STEP * (n_chunks - 1) <= O::CHUNK)
+        chunk = chunk / STEP * STEP;
     const uint32_t c_first = 2 * part;
     const uint32_t c_end = n_parts < octet_parts<O>(n_bin) - part ? 2 * (part + n_parts) : n_chunks;
     __shared__ float s_scale[8], s_iscale[8];
