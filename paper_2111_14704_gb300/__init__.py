@@ -446,8 +446,14 @@ def _field_args(modes, u_gas):
         rec[:, 3:6] = modes["e"]
         rec[:, 6] = modes["amp"]
         rec[:, 7] = modes["phase"]
-        buf[8 * nm:9 * nm] = np.asarray(modes["sigma"], dtype=np.float64).reshape(-1)[:nm]
-    buf[9 * nm:9 * nm + 3] = np.asarray(u_gas, dtype=np.float64).reshape(-1)[:3]
+        sigma = np.asarray(modes["sigma"], dtype=np.float64).reshape(-1)
+        if sigma.size < nm:  # (numpy would spread a single value over all modes)
+            raise ValueError(f"{sigma.size} values of sigma for {nm} modes")
+        buf[8 * nm:9 * nm] = sigma[:nm]
+    gas = np.asarray(u_gas, dtype=np.float64).reshape(-1)
+    if gas.size < 3:
+        raise ValueError(f"u_gas has {gas.size} components, needs 3")
+    buf[9 * nm:] = gas[:3]
     return buf, C.addressof(C.c_double.from_buffer(buf)), nm
 
 
