@@ -19,8 +19,9 @@
 
 namespace rsol {
 
-template <typename T, int SHAPE, int B, int NW>
+template <int SHAPE, int B, int NW>
 struct MomCfg {
+    using T = double;
     static constexpr int NP = SHAPE == 1 ? 2 : 3;
     static constexpr int NS = NP * NP * NP;
     static constexpr int TE = B + 4;
@@ -53,10 +54,11 @@ __device__ __forceinline__ void state_moments(const MomArgs<T> &a, T w, const T 
         Q[5 + q] = N * a.qc * (u[q] * ig);
 }
 
-template <typename T, int SHAPE, int B, int NW>
-__global__ void __launch_bounds__(NW * 32) moments_binned_kernel(MomArgs<T> a, BinGeom g)
+template <int SHAPE, int B, int NW>
+__global__ void __launch_bounds__(NW * 32) moments_binned_kernel(MomArgs<double> a, BinGeom g)
 {
-    using Cfg = MomCfg<T, SHAPE, B, NW>;
+    using T = double;
+    using Cfg = MomCfg<SHAPE, B, NW>;
     constexpr int TE = Cfg::TE, RS = Cfg::RS, PS = Cfg::PS, TN = Cfg::TN;
     constexpr int NP = Cfg::NP, NS = Cfg::NS, WS = Cfg::WS, QO = Cfg::QO;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -625,9 +627,9 @@ cudaError_t launch_moments_binned(const MomArgs<T> &a, const BinGeom &g, int64_t
         return cudaGetLastError();
     } else {
         constexpr int NW = B == 8 ? 8 : 16;  // 8^3 tiles: fewer warps fit
-        using Cfg = MomCfg<T, SHAPE, B, NW>;
+        using Cfg = MomCfg<SHAPE, B, NW>;
         static_assert(Cfg::smem_bytes <= 232448 - 1024, "moments tiles exceed shared memory");
-        auto kern = moments_binned_kernel<T, SHAPE, B, NW>;
+        auto kern = moments_binned_kernel<SHAPE, B, NW>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              int(Cfg::smem_bytes));
         if (e != cudaSuccess)

@@ -184,11 +184,6 @@ __device__ __forceinline__ void sts_node(double *p, const double F[6])
     reinterpret_cast<double2 *>(p)[2] = make_double2(F[4], F[5]);
 }
 
-__device__ __forceinline__ void store_q8(float *p, const float Q[8])
-{
-    reinterpret_cast<float4 *>(p)[0] = make_float4(Q[0], Q[1], Q[2], Q[3]);
-    reinterpret_cast<float4 *>(p)[1] = make_float4(Q[4], Q[5], Q[6], Q[7]);
-}
 __device__ __forceinline__ void store_q8(double *p, const double Q[8])
 {
 #pragma unroll
@@ -196,15 +191,6 @@ __device__ __forceinline__ void store_q8(double *p, const double Q[8])
         reinterpret_cast<double2 *>(p)[q / 2] = make_double2(Q[q], Q[q + 1]);
 }
 // one packet's stencil weights into its padded staging row (16-byte stores)
-template <int WS, int NS>
-__device__ __forceinline__ void store_wrow(float *p, const float (&W)[NS])
-{
-#pragma unroll
-    for (int k = 0; k < WS; k += 4)
-        reinterpret_cast<float4 *>(p)[k / 4] =
-            make_float4(W[k], k + 1 < NS ? W[k + 1] : 0.f, k + 2 < NS ? W[k + 2] : 0.f,
-                        k + 3 < NS ? W[k + 3] : 0.f);
-}
 template <int WS, int NS>
 __device__ __forceinline__ void store_wrow(double *p, const double (&W)[NS])
 {
@@ -215,38 +201,10 @@ __device__ __forceinline__ void store_wrow(double *p, const double (&W)[NS])
 
 // the N densities of a phase-2 lane role, starting at p (N = 8: all; N = 2: a pair)
 template <int N>
-__device__ __forceinline__ void load_qpart(const float *p, float Q[N])
-{
-    if constexpr (N == 8) {
-        const float4 a = reinterpret_cast<const float4 *>(p)[0];
-        const float4 b = reinterpret_cast<const float4 *>(p)[1];
-        Q[0] = a.x; Q[1] = a.y; Q[2] = a.z; Q[3] = a.w; Q[4] = b.x; Q[5] = b.y; Q[6] = b.z; Q[7] = b.w;
-    } else {
-        const float2 a = *reinterpret_cast<const float2 *>(p);
-        Q[0] = a.x; Q[1] = a.y;
-    }
-}
-template <int N>
 __device__ __forceinline__ void load_qpart(const double *p, double Q[N])
 {
 #pragma unroll
     for (int q = 0; q < N; q += 2) {
-        const double2 v = reinterpret_cast<const double2 *>(p)[q / 2];
-        Q[q] = v.x;
-        Q[q + 1] = v.y;
-    }
-}
-
-__device__ __forceinline__ void load_q8(const float *p, float Q[8])
-{
-    const float4 a = reinterpret_cast<const float4 *>(p)[0];
-    const float4 b = reinterpret_cast<const float4 *>(p)[1];
-    Q[0] = a.x; Q[1] = a.y; Q[2] = a.z; Q[3] = a.w; Q[4] = b.x; Q[5] = b.y; Q[6] = b.z; Q[7] = b.w;
-}
-__device__ __forceinline__ void load_q8(const double *p, double Q[8])
-{
-#pragma unroll
-    for (int q = 0; q < 8; q += 2) {
         const double2 v = reinterpret_cast<const double2 *>(p)[q / 2];
         Q[q] = v.x;
         Q[q + 1] = v.y;
@@ -315,9 +273,9 @@ __device__ __forceinline__ void origin_cursors(const int *hist, int *cursor, int
 // (largest axis weights for that offset: CIC 1, 1; TSC 1/2, 3/4, 1/2 per
 // axis).  The weights are per-axis products, so the sum is three 3-tap passes
 // along x, y and z, one tile row per thread and pass; exact in float (the terms
-// are small integers times products of 1/2 and 3/4).  scratch holds 2 TE^3
-// floats.  Returns this thread's largest node value (reduce over the CTA);
-// ends with scratch still in use by no thread, but without a final barrier.
+// are small integers times products of 1/2 and 3/4).  One pass per call, 0 to 2, all
+// threads, with a barrier between the calls; scratch holds 2 TE^3 floats.  Pass 2 raises
+// gmax to this thread's largest node value (reduce over the CTA).
 template <int SHAPE, int TE, int RS, int PS, typename Hist>
 __device__ __forceinline__ void weight_bound_pass(int pass, Hist hist, float *scratch, float &gmax)
 {
@@ -348,18 +306,6 @@ __device__ __forceinline__ void weight_bound_pass(int pass, Hist hist, float *sc
         }
     }
 }
-template <int SHAPE, int TE, int RS, int PS, typename Hist>
-__device__ __forceinline__ float tile_weight_bound(Hist hist, float *scratch)
-{
-    float gmax = 0.f;
-    weight_bound_pass<SHAPE, TE, RS, PS>(0, hist, scratch, gmax);
-    __syncthreads();
-    weight_bound_pass<SHAPE, TE, RS, PS>(1, hist, scratch, gmax);
-    __syncthreads();
-    weight_bound_pass<SHAPE, TE, RS, PS>(2, hist, scratch, gmax);
-    return gmax;
-}
-
 // Few packets: staging and flushing the tiles would cost more than the
 // packets' own global-memory gathers and atomics.
 template <typename T, int SHAPE, bool DET>
@@ -394,12 +340,13 @@ __device__ __forceinline__ void tile_axes(int *axis, int ox, int oy, int oz, int
     }
 }
 
-// The work of one CTA on one bin: packets [lo, hi) of the bin whose anchors
+// The work of one CTA on one bin (FP64): packets [lo, hi) of the bin whose anchors
 // were in bin (bx, by, bz) of the box described by a at the last sort.
-template <typename T, int SHAPE, int B, int NW, bool DET>
-__device__ __forceinline__ void binned_cta(const PushArgs<T> &a, uint32_t lo, uint32_t hi,
+template <int SHAPE, int B, int NW, bool DET>
+__device__ __forceinline__ void binned_cta(const PushArgs<double> &a, uint32_t lo, uint32_t hi,
                                            int bx, int by, int bz)
 {
+    using T = double;
     using Cfg = BinnedCfg<T, SHAPE, B, NW, DET>;
     using Acc = typename Cfg::Acc;
     constexpr int TE = Cfg::TE, RS = Cfg::RS, PS = Cfg::PS, TN = Cfg::TN;
@@ -1181,7 +1128,7 @@ __device__ __forceinline__ void tile_cta(const PushArgs<T> &a, uint32_t lo, uint
     if constexpr (kUsesOctets<T>)
         octet_cta<SHAPE, B, NW, DET>(a, lo, hi, bx, by, bz, part, n_parts, tmap);
     else
-        binned_cta<T, SHAPE, B, NW, DET>(a, lo, hi, bx, by, bz);
+        binned_cta<SHAPE, B, NW, DET>(a, lo, hi, bx, by, bz);
 }
 
 template <typename T, int SHAPE, int B, int NW, bool DET>
