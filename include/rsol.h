@@ -119,7 +119,8 @@ const char *rsol_last_error(const rsol_ctx *ctx);
  * eight feedback densities into d_feedback when it is not NULL, drift x.
  * Updates parts->cell, off and u in place; w is read only.  dt > 0.  When
  * parts is the set the last rsol_sort wrote, the binned shared-memory kernel
- * runs; otherwise a kernel that needs no ordering runs (same results up to
+ * runs (FP32 sets that are sparse on many bins: after a kernel for their bins of
+ * at most 768 packets); otherwise a kernel that needs no ordering runs (same results up to
  * the order of floating-point additions; deterministic mode makes each of
  * them bitwise reproducible from run to run).  "The set the last rsol_sort
  * wrote" is decided by buffer identity: parts->cell and parts->n equal the
@@ -136,7 +137,8 @@ rsol_status rsol_push_gather(rsol_ctx *ctx, const rsol_particles *parts,
 /*
  * State moments at the current positions and momenta (Sec. 2 packet totals
  * N_j, P_j = N_j m c u, E_j = N_j gamma m c^2, per unit volume, plus the
- * current N_j q c beta), deposited with W into d_moments (accumulated).
+ * current N_j q c beta), deposited with W into d_moments (accumulated).  A
+ * packet with a value that is not finite changes only the nodes of its stencil.
  */
 rsol_status rsol_deposit(rsol_ctx *ctx, const rsol_particles *parts, void *d_moments,
                          void *stream);
@@ -331,12 +333,15 @@ rsol_status rsol_push_subcycled(rsol_ctx *ctx, const rsol_particles *parts, cons
  * rsol_sort; then, for each sub-step s = 0 .. 2^top - 1 of the highest level
  * present, every level k whose step ends there (s a multiple of 2^(top - k))
  * advances by one binned launch over its own bins, with h, c~ dt/dx and the
- * deposit scaled by 2^-k.  `out` holds the advanced packets in that order; in and out
+ * deposit scaled by 2^-k.  (A FP32 level none of whose 8^3 bins holds more than
+ * 768 packets may take the order-free kernel instead where that is expected to be
+ * faster, with warps = 0 and deterministic = 0: the same packet bits, sums of the
+ * same kind as the binned kernel's in such bins.)  `out` holds the advanced packets in that order; in and out
  * must not share arrays.  Needs the context's bin to be 4 or 8, c~ dt/dx <= 1
  * (the tiles' 2-node halo covers one cell of drift over the step) and
  * (max_level + 1) x bins x bin^3 < 2^31.  h_level_counts (host, max_level + 1
  * int64, may be NULL) receives the packets per level.  Synchronises the stream
- * once, after the sort, to read the level counts.
+ * once, after the sort, to read the level counts and each level's fullest bin.
  */
 rsol_status rsol_sort_push_subcycled(rsol_ctx *ctx, const rsol_particles *in, rsol_particles *out,
                                      const void *d_fields, double dt, const rsol_subcycle_desc *desc,

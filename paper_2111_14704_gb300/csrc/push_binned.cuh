@@ -69,13 +69,14 @@ __host__ __device__ constexpr uint32_t sparse_cta_limit()
 template <int SHAPE, int B, bool DET>
 __host__ __device__ constexpr uint32_t sliced_cta_limit(uint32_t slices)
 {
-    const uint32_t limit = sparse_cta_limit<SHAPE, B, DET>(), most = B == 8 ? 768u : 256u;
+    const uint32_t limit = sparse_cta_limit<SHAPE, B, DET>(), most = B == 8 ? kGlobalBinMost : 256u;
     return DET ? limit : limit * slices < most ? limit * slices : most;
 }
 
 struct BinGeom {
     const uint32_t *bin_start;
     int nbx, nby, nbz;
+    uint32_t skip = 0;  // push: bins of at most this many packets are another kernel's
 };
 
 template <typename T, int SHAPE, int B, int NW, bool DET>
@@ -1150,8 +1151,10 @@ __global__ void __launch_bounds__(NW * 32)
         prefetch_l2(a.u2, plo, phi);
         prefetch_l2(a.w, plo, phi);
     }
-    const uint32_t lo = g.bin_start[bin], hi = g.bin_start[bin + 1];
+    const uint32_t lo = g.bin_start[bin];
+    uint32_t hi = g.bin_start[bin + 1];
     if constexpr (kUsesOctets<T>) {
+        hi = hi - lo <= g.skip ? lo : hi;  // (an early return here cost CIC bins 4 %)
         if (gridDim.y > 1) {  // a sparse bin in slices; a dense one is the first slice's
             const uint32_t n = hi - lo, slice = blockIdx.y;
             if (n <= sliced_cta_limit<SHAPE, B, DET>(gridDim.y)) {
@@ -1169,6 +1172,27 @@ __global__ void __launch_bounds__(NW * 32)
         }
     }
     tile_cta<T, SHAPE, B, NW, DET>(a, lo, hi, bx, by, bz, 0, 0xFFFFFFFFu, use_tma ? &tmap : nullptr);
+}
+
+// The bins of at most kGlobalBinMost packets of one box, a CTA per kSplitShare packets: for
+// sets sparse on many bins, where a CTA with tiles per bin leaves each SM one bin's few
+// packets to wait for.  A denser bin is left to push_binned_kernel, launched after it, so
+// that crowded packets keep their tile's accuracy.
+constexpr int kSplitShare = 128;
+template <int SHAPE>
+__global__ void __launch_bounds__(kSplitShare) push_sparse_bins_kernel(const __grid_constant__ PushArgs<float> a,
+                                                                       const uint32_t *__restrict__ bin_start)
+{
+    const uint32_t lo = bin_start[blockIdx.x], n = bin_start[blockIdx.x + 1] - lo;
+    const uint32_t i = blockIdx.y * kSplitShare + threadIdx.x;
+    if (n > kGlobalBinMost || i >= n)
+        return;
+    int flag = 0;
+    auto gather_global = [&](int64_t node, float F[6]) { load_node(a.fields + node * 8, F); };
+    auto deposit_global = [&](int64_t node, float W, const float Q[8]) { red_node(a.fb + node * 8, W, Q); };
+    push_one<float, SHAPE, true>(a, int64_t(lo) + i, gather_global, deposit_global, &flag);
+    if (flag)
+        atomicOr(a.status, flag);
 }
 
 // One box of a batch: grid, node offset into the concatenated grids, first
@@ -1405,6 +1429,17 @@ cudaError_t push_binned_dispatch(const PushDesc &d, cudaStream_t s)
     BinGeom g{d.bin_start, d.nbx, d.nby, d.nbz};
     const int nbins = d.nbx * d.nby * d.nbz;
     const bool det = d.det != 0;
+    if constexpr (kUsesOctets<T>) {
+        if (d.split) {
+            const dim3 grid{unsigned(nbins), unsigned((kGlobalBinMost + kSplitShare - 1) / kSplitShare)};
+            auto kern = d.shape == 1 ? push_sparse_bins_kernel<1> : push_sparse_bins_kernel<2>;
+            kern<<<grid, kSplitShare, 0, s>>>(a, d.bin_start);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess)
+                return e;
+            g.skip = kGlobalBinMost;
+        }
+    }
 #define RSOL_BINNED(SH, BB)                                                                  \
     return det ? launch_binned<T, SH, BB, true>(a, g, nbins, d.sm_count, d.warps, s)        \
                : launch_binned<T, SH, BB, false>(a, g, nbins, d.sm_count, d.warps, s)

@@ -192,11 +192,12 @@ rsol_status rsol_push_gather(rsol_ctx *ctx, const rsol_particles *P, const void 
     if (ctx->sorted_cell == P->cell && ctx->sorted_n == P->n) {
         d.bin_start = ctx->sort.bin_start;
         d.tile_mode = 1;
+        d.split = d_feedback && split_faster(ctx, P->n);
     }
     cudaError_t e = ctx->p.precision == 32 ? rsol::push_f32(d, s) : rsol::push_f64(d, s);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "rsol_push_gather launch");
-    ctx->launches += 1 + (det ? 1 : 0);
+    ctx->launches += 1 + (det ? 1 : 0) + (d.split ? 1 : 0);
     if (det) {
         e = ctx->p.precision == 32
                 ? rsol::fixed_to_grid_f32(ctx->fx, d_feedback, n_nodes(ctx) * 8, 1.0 / ctx->fx_scale,

@@ -26,6 +26,7 @@ struct PushDesc {
     int bin, nbx, nby, nbz;
     int warps;              // binned kernel CTA width: 8, or 0 / 16 for the widest that fits
     int tile_mode;          // 0 = order-free kernel; 1 = binned shared-memory kernel
+    int split;              // binned, FP32, 8^3 bins: sparse bins by a kernel of their own, first
 };
 
 struct MomentsDesc {
@@ -75,6 +76,8 @@ struct LossDesc {
 cudaError_t losses_f32(const LossDesc &d, cudaStream_t s);
 cudaError_t losses_f64(const LossDesc &d, cudaStream_t s);
 cudaError_t push_f32(const PushDesc &d, cudaStream_t s);
+// Most packets of an 8^3 bin that any FP32 push sums by global atomics.
+constexpr uint32_t kGlobalBinMost = 768;
 // CTAs that a box of few bins deals a sparse bin to (FP32; at most one CTA per SM).
 inline int bin_slices(int sm_count, int64_t nbins)
 {

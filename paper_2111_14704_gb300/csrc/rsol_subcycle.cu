@@ -41,29 +41,16 @@ __global__ void __launch_bounds__(256) level_summary_kernel(const uint32_t *__re
 }
 
 // Whether a FP32 level of n packets goes through the order-free kernel: only where no
-// bin holds more than the 768 packets that the binned kernel too sums in global FP32
-// (sliced_cta_limit), so that which kernel runs costs no accuracy, and only where it is
-// expected to be faster.  From one GB300, 8^3 bins, us per push, p packets per bin:
-//   order-free             max(12.5, 5 + 0.31e-3 n) TSC, max(5.2, 4 + 0.08e-3 n) CIC
-//   binned, per wave       10 + 0.07 p / slices TSC, 6.2 + 0.018 p / slices CIC in sparse
-//                          bins (160, 384 packets a slice); 11 + 9.5e-3 p, 10.5 + 3e-3 p in tiles
-// (binned / order-free, TSC: 16^3 nodes x 4096 packets 11.4 / 10.9, 40^3 x 16000 20.5 / 13.8,
-// 48^3 x 55296 26.8 / 23.4, 48^3 x 110592 32.2 / 41.4, 64^3 x 65536 71.5 / 24.2, x 262144
-// 63.3 / 80.5; CIC: 16^3 x 4096 6.2 / 4.9, 64^3 x 262144 47.2 / 24.8.)  A caller who asks
-// for a CTA width asks for the binned kernel.
+// bin holds more than the kGlobalBinMost packets that the binned kernel too sums in global
+// FP32, so that which kernel runs costs no accuracy, and only where it is expected to be
+// faster.  A caller who asks for a CTA width asks for the binned kernel.
 bool order_free_faster(const rsol_ctx *ctx, int64_t n, uint32_t fullest)
 {
-    if (ctx->p.precision != 32 || ctx->p.deterministic || ctx->bin != 8 || ctx->p.warps != 0 || fullest > 768)
+    if (ctx->p.precision != 32 || ctx->p.deterministic || ctx->bin != 8 || ctx->p.warps != 0 ||
+        fullest > rsol::kGlobalBinMost)
         return false;
-    const bool cic = ctx->p.shape == 1;
-    const double p = double(n) / double(ctx->nbins);
-    const int slices = rsol::bin_slices(ctx->sm_count, ctx->nbins);
-    const double waves = double((ctx->nbins + ctx->sm_count - 1) / ctx->sm_count);
-    const bool sparse = p <= double((cic ? 384 : 160) * slices);
-    const double binned = sparse ? (cic ? 6.2 + 0.018 * p / slices : 10.0 + 0.07 * p / slices)
-                                 : (cic ? 10.5 + 3e-3 * p : 11.0 + 9.5e-3 * p);
-    const double free = cic ? std::fmax(5.2, 4.0 + 0.08e-3 * n) : std::fmax(12.5, 5.0 + 0.31e-3 * n);
-    return free < waves * binned;
+    const PushEstimate e = push_estimate(ctx, n);
+    return e.order_free < e.binned;
 }
 
 } // namespace
