@@ -62,10 +62,10 @@ LOSS_BYTES_PER_PACKET = 36
 # the same packets per cell, so the same bytes per packet), and the hash of the
 # kernel sources it was taken on: the bench reports traffic only while the
 # sources still match.
-NCU_TRAFFIC_PER_PACKET = (345.784832e6 + 216.639744e6) / (1 << 23)
+NCU_TRAFFIC_PER_PACKET = (345.294592e6 + 217.086720e6) / (1 << 23)
 # warp instructions the same capture counted per packet (smsp__inst_executed.sum / packets)
-NCU_INST_PER_PACKET = 332508052 / (1 << 23)
-NCU_SOURCE_HASH = "f00774e269f09e18"
+NCU_INST_PER_PACKET = 332752572 / (1 << 23)
+NCU_SOURCE_HASH = "69044991049cfd9b"
 # instruction issue peak: 152 SMs x 4 schedulers x one warp instruction per clock
 ISSUE_SCHEDULERS = 152 * 4
 
