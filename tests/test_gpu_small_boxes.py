@@ -86,8 +86,12 @@ def test_dense_bins_keep_the_accuracy_of_tiles(edge, shape, n, crowded):
 
 def test_a_crowded_bin_of_a_sub_cycled_level_keeps_the_accuracy_of_tiles():
     """About 20000 packets in one cell of 64^3, few for the box: a level of more than 768
-    of them takes the tiles, two chunks a sum, in each of its 2^k sub-steps.  (Packets
-    whose limits lie within 1e-3 of a level's edge are left out.)"""
+    of them takes the tiles, so rho is as near the oracle's as with the tiles asked for (16
+    warps), up to the order of the additions.  Tiles make 28 additions on a node, global
+    sums 111,000, whose rms rounding is sqrt(111000 / 28) = 63 times as large; the bar is the
+    geometric middle, 8.  (The sub-steps add nearly equal values, whose roundings are not
+    independent: no bar from their number alone.  Packets whose limits lie within 1e-3 of a
+    level's edge are left out.)"""
     grid, dt = (64, 64, 64), 10.0
     parts = ri.make_particles(20400, grid, 67)
     parts["cell"][:] = 11
@@ -96,14 +100,15 @@ def test_a_crowded_bin_of_a_sub_cycled_level_keeps_the_accuracy_of_tiles():
     r = np.log2(dt / oracle.dt_limits(op, planes, oracle.Particles(parts), 0.2))
     keep = np.abs(r - np.round(r)) > 1e-3
     parts = {k: np.ascontiguousarray(v[..., keep]) for k, v in parts.items()}
-    ctx = rs.Context(rs.Params(*grid, shape=2, precision=32, c_tilde=0.1))
-    P, fb = rs.Particles.from_numpy(parts, 32), ctx.grid_tensor()
-    counts = ctx.sort_push_subcycled(P, rs.Particles.empty(P.n, 32), rs.fields_to_device(planes, 32), dt, 0.2, fb)
-    ctx.check()
     G, levels = oracle.step_subcycled(op, planes, oracle.Particles(parts), 0.2)
-    assert np.array_equal(counts, np.bincount(levels, minlength=len(counts)))
-    adds = sum(2**k * (c if c <= 768 else math.ceil(c / 4352)) for k, c in enumerate(counts))
-    got = rs.grid_to_planes(fb)
-    assert rel_l2(got[0], G[0]) <= bar(adds)
-    for q in range(1, 8):
-        assert rel_l2(got[q], G[q]) <= 1e-5, q
+    err = []
+    for warps in (0, 16):
+        ctx = rs.Context(rs.Params(*grid, shape=2, precision=32, c_tilde=0.1, warps=warps))
+        P, fb = rs.Particles.from_numpy(parts, 32), ctx.grid_tensor()
+        counts = ctx.sort_push_subcycled(P, rs.Particles.empty(P.n, 32), rs.fields_to_device(planes, 32), dt, 0.2,
+                                         fb)
+        ctx.check()
+        assert np.array_equal(counts, np.bincount(levels, minlength=len(counts)))
+        err.append([rel_l2(x, y) for x, y in zip(rs.grid_to_planes(fb), G)])
+    assert err[0][0] <= 8 * err[1][0]
+    assert max(err[0]) <= 1e-5
